@@ -1,9 +1,11 @@
 // k_index.cu -- index construction on the device: position updates, Morton
-// keys, onesweep radix sort of the objects, and PR-quadtree leaves.
+// keys, radix sort of the objects, and PR-quadtree leaves.
 //
 // Paper steps: batch processing of updates (Sec. 2.2), Alg. 1
 // (GPUcalculateMortonHash, GPUradixSort, GPUdetectQuadrants +
 // CPUcheckQuadrants), uniform grid indexing (Sec. 5.2).
+#include <cstddef>
+
 #include "mqr_internal.cuh"
 
 namespace mqr {
@@ -70,323 +72,632 @@ void launch_state_stamps(cudaStream_t st, const uint8_t *present, uint32_t nmax,
 }
 
 // ---------------------------------------------------------------------------
-// a2: Morton keys at l_max = 15 of every slot, fused with the digit
-// histograms of the four 8-bit passes of the object sort (bits 32..63 of the
-// packed key), the first pass's per-tile digit counts (a block covers exactly
-// one sort tile) and the count of present objects.
+// The start of a tick: clears the arena (bytes a multiple of 16, Info first)
+// and takes over the update kernels' error bits (upd_err) or, for a slot, the
+// snapshot's counters and error bits (snap: n_present, n_leaves, max_level,
+// err).  One launch instead of a memset and two or three small copies, each of
+// which cost a dependent step of about 2 us on the stream.
 // ---------------------------------------------------------------------------
-constexpr int kMortonThreads = 256, kMortonItems = 16;
-static_assert(kMortonThreads * kMortonItems == kSortTile, "a Morton block is one sort tile");
+__global__ void __launch_bounds__(256)
+tick_begin_kernel(uint4 *__restrict__ arena, size_t n16, unsigned long long *upd_err,
+                  const unsigned long long *__restrict__ snap) {
+    constexpr size_t kInfo16 = (sizeof(Info) + 15) / 16;
+    const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    for (size_t i = i0; i < n16; i += (size_t)gridDim.x * blockDim.x)
+        if (i >= kInfo16) arena[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (i0 < sizeof(Info) / 8) {
+        unsigned long long v = 0;
+        if (i0 == offsetof(Info, err) / 8) {
+            v = snap ? snap[3] : *upd_err;
+            if (!snap) *upd_err = 0;
+        } else if (snap && i0 < 3) {
+            v = snap[i0];
+        }
+        reinterpret_cast<unsigned long long *>(arena)[i0] = v;
+    }
+}
 
-__global__ void __launch_bounds__(kMortonThreads)
+void launch_tick_begin(cudaStream_t st, void *arena, size_t bytes, unsigned long long *upd_err,
+                       const unsigned long long *snap) {
+    static_assert(offsetof(Info, n_present) == 0 && offsetof(Info, n_leaves) == 8 && offsetof(Info, max_level) == 16 &&
+                      sizeof(Info) <= 256 * 8, "the counters a snapshot hands over, and one block for Info");
+    const size_t n16 = bytes / 16;
+    const unsigned grid = (unsigned)((n16 + 1023) / 1024 < 304 ? (n16 + 1023) / 1024 : 304);
+    tick_begin_kernel<<<grid ? grid : 1, 256, 0, st>>>(reinterpret_cast<uint4 *>(arena), n16, upd_err, snap);
+}
+
+constexpr uint32_t kSortDirectGroups = 32;      // tiles add up to this many group rows themselves (see a3)
+
+// A tile's count of one digit into the coarse rows (layout: see a3).
+__device__ __forceinline__ void add_digit_count(uint32_t *group_counts, uint32_t tile, uint32_t d, uint32_t c,
+                                                uint32_t n) {
+    atomicAdd(group_counts + (size_t)(kSortTotalRows + tile / kSortGroup) * 256 + d, c);
+    if (sort_groups(n) <= kSortDirectGroups) atomicAdd(group_counts + (tile % kSortTotalRows) * 256 + d, c);
+}
+
+// ---------------------------------------------------------------------------
+// a2: Morton keys at l_max = 15 of every slot, fused with the first sort
+// pass's digit counts (a block covers exactly one sort tile) and the count of
+// present objects.  Bound by memory: 16 B read and 8 B written per slot (18 us
+// at 4M slots, 5.3 TB/s; 24 with counts of all four digits; 105 -> 59 at 12M
+// slots of 256 worlds, each block searching the worlds of its ends only).
+// stamp may be null: every object is present (info may then be null too).
+// ---------------------------------------------------------------------------
+constexpr int kMortonBatch = 4;           // slots of a thread in flight (eight at 2 blocks per SM: 36 us against 26 at 4M)
+
+__global__ void __launch_bounds__(kSortThreads, 3)
 morton_kernel(const float2 *__restrict__ pos, const unsigned long long *__restrict__ stamp,
               uint32_t nmax, float x0, float y0, float sx, float sy, Worlds worlds,
-              unsigned long long *__restrict__ keys, uint32_t *__restrict__ hist,
-              uint32_t *__restrict__ tile_counts, Info *info) {
-    __shared__ uint32_t s_hist[4 * 256];
-    __shared__ uint32_t s_tile[256];              // this tile's counts of the first digit
-    __shared__ uint32_t s_cnt;
-    for (int i = threadIdx.x; i < 4 * 256; i += kMortonThreads) s_hist[i] = 0;
-    for (int i = threadIdx.x; i < 256; i += kMortonThreads) s_tile[i] = 0;
-    if (threadIdx.x == 0) s_cnt = 0;
+              unsigned long long *__restrict__ keys, uint32_t *__restrict__ tile_counts,
+              uint32_t *__restrict__ group_counts, Info *info) {
+    __shared__ uint32_t s_hist[256];
+    __shared__ uint32_t s_cnt, s_w[2];
+    const int tid = threadIdx.x;
+    const uint32_t base = blockIdx.x * kSortTile;
+    if (tid < 256) s_hist[tid] = 0;
+    if (tid == 256) s_cnt = 0;
+    if (worlds.n && tid < 64) {                        // the worlds of the block's first and last slot
+        const uint32_t w = world_of_warp(tid < 32 ? base : min(base + kSortTile, nmax) - 1u, worlds.obj_base, worlds.n);
+        if ((tid & 31) == 0) s_w[tid >> 5] = w;
+    }
     __syncthreads();
+    const uint32_t w0 = worlds.n ? s_w[0] : 0u, w1 = worlds.n ? s_w[1] + 1u : 0u;
     uint32_t present = 0;
-    const uint32_t base = blockIdx.x * (kMortonThreads * kMortonItems);
-#pragma unroll 4
-    for (int it = 0; it < kMortonItems; ++it) {
-        uint32_t i = base + it * kMortonThreads + threadIdx.x;
-        if (i >= nmax) break;
-        uint32_t k;
-        if (stamp[i] != 0ull) {
-            float2 p = pos[i];
-            uint32_t ci = cell_of(p.x, x0, sx), cj = cell_of(p.y, y0, sy);
-            if (worlds.n) {
-                const uint32_t w = world_of(i, worlds.obj_base, worlds.n);
-                ci = world_cell(ci, w, worlds.bits, 0);
-                cj = world_cell(cj, w, worlds.bits, 1);
+#pragma unroll 1
+    for (int b = 0; b < kSortItems; b += kMortonBatch) {
+        float2 p[kMortonBatch];
+        unsigned long long st[kMortonBatch];
+#pragma unroll
+        for (int it = 0; it < kMortonBatch; ++it) {
+            const uint32_t i = base + (b + it) * kSortThreads + tid;
+            if (i < nmax) {
+                p[it] = __ldg(pos + i);
+                st[it] = stamp ? __ldg(stamp + i) : 1ull;
             }
-            k = morton2(ci, cj);
-            ++present;
-        } else {
-            k = kAbsentKey;
         }
-        keys[i] = ((unsigned long long)k << 32) | i;
-        atomicAdd(&s_tile[k & 255u], 1u);
-        atomicAdd(&s_hist[0 * 256 + (k & 255u)], 1u);
-        atomicAdd(&s_hist[1 * 256 + ((k >> 8) & 255u)], 1u);
-        atomicAdd(&s_hist[2 * 256 + ((k >> 16) & 255u)], 1u);
-        atomicAdd(&s_hist[3 * 256 + (k >> 24)], 1u);
+#pragma unroll
+        for (int it = 0; it < kMortonBatch; ++it) {
+            const uint32_t i = base + (b + it) * kSortThreads + tid;
+            if (i >= nmax) break;
+            uint32_t k = kAbsentKey;
+            if (st[it] != 0ull) {
+                uint32_t ci = cell_of(p[it].x, x0, sx), cj = cell_of(p[it].y, y0, sy);
+                if (worlds.n) {
+                    const uint32_t w = world_of(i, worlds.obj_base, w0, w1);
+                    ci = world_cell(ci, w, worlds.bits, 0);
+                    cj = world_cell(cj, w, worlds.bits, 1);
+                }
+                k = morton2(ci, cj);
+                ++present;
+            }
+            keys[i] = ((unsigned long long)k << 32) | i;
+            atomicAdd(&s_hist[k & 255u], 1u);
+        }
     }
     present = warp_sum(present);
-    if ((threadIdx.x & 31) == 0 && present) atomicAdd(&s_cnt, present);
+    if ((tid & 31) == 0 && present) atomicAdd(&s_cnt, present);
     __syncthreads();
-    for (int i = threadIdx.x; i < 4 * 256; i += kMortonThreads)
-        if (s_hist[i]) atomicAdd(hist + i, s_hist[i]);
-    const uint32_t tiles = (nmax + kSortTile - 1) / kSortTile;
-    for (int i = threadIdx.x; i < 256; i += kMortonThreads) tile_counts[(size_t)i * tiles + blockIdx.x] = s_tile[i];
-    if (threadIdx.x == 0 && s_cnt) atomicAdd(&info->n_present, (unsigned long long)s_cnt);
+    if (tid < 256) {
+        const uint32_t c = s_hist[tid];
+        tile_counts[(size_t)blockIdx.x * 256 + tid] = c;
+        if (c) add_digit_count(group_counts, blockIdx.x, tid, c, nmax);
+    }
+    if (info && tid == 0 && s_cnt) atomicAdd(&info->n_present, (unsigned long long)s_cnt);
 }
 
 void launch_morton_keys(cudaStream_t st, const float2 *pos, const unsigned long long *stamp,
                         uint32_t nmax, float x0, float y0, float sx, float sy, Worlds worlds,
-                        unsigned long long *keys, uint32_t *hist4x256, uint32_t *tile_counts, Info *info) {
+                        unsigned long long *keys, uint32_t *tile_counts, uint32_t *group_counts, Info *info) {
     if (nmax == 0) return;
-    uint32_t per = kMortonThreads * kMortonItems;
-    morton_kernel<<<(nmax + per - 1) / per, kMortonThreads, 0, st>>>(pos, stamp, nmax, x0, y0, sx, sy,
-                                                                      worlds, keys, hist4x256, tile_counts,
-                                                                      info);
+    morton_kernel<<<sort_tiles(nmax), kSortThreads, 0, st>>>(pos, stamp, nmax, x0, y0, sx, sy, worlds, keys,
+                                                             tile_counts, group_counts, info);
 }
 
 // ---------------------------------------------------------------------------
-// Generic digit histograms (up to 8 passes) for the other sorts.
+// a3: one pass of a stable LSD radix sort (8-bit digit at `shift`): per-tile
+// digit counts, then a rank-and-scatter kernel that finds the start of every
+// tile's digit runs from those counts, so no tile waits for another.
+//
+// Digit counts, rows of 256 adjacent words: tile_counts[t][d] for every tile
+// of kSortTile keys; group_counts: kSortTotalRows rows that add up to the
+// digits' totals, then a row for every kSortGroup tiles (zeroed by the caller,
+// accumulated by the counting kernels; one row of totals met 1,000 additions
+// per word at 4M keys: tile counts 9.4 us against 6).  A tile's run of digit d starts at
+//   digit start(d) + sum of the rows of earlier groups
+//                  + sum of tile_counts[t'][d], t' < t in the same group,
+// the digit starts being the scan of the totals.
+// Up to kSortDirectGroups groups the tile adds the rows itself (coalesced,
+// independent loads); above, group_scan_kernel turns the group rows into
+// starts first, so that a tile never reads more than kSortGroup rows.
+//
+// Measured, all four passes with their counts (start: tile counts, a scan
+// kernel per digit over the tiles, match-any ranking): 0.089 -> 0.061 ms at
+// 1M objects, 0.209 -> 0.149 ms at 4M, 0.534 -> 0.367 ms at 12M.
 // ---------------------------------------------------------------------------
-struct Shifts { int s[8]; int n; };
 
-__global__ void __launch_bounds__(256)
-hist_kernel(const unsigned long long *__restrict__ keys, uint32_t n, Shifts sh, uint32_t *hist) {
-    __shared__ uint32_t s_hist[8 * 256];
-    for (int i = threadIdx.x; i < sh.n * 256; i += 256) s_hist[i] = 0;
-    __syncthreads();
-    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-        unsigned long long k = keys[i];
-        for (int d = 0; d < sh.n; ++d) atomicAdd(&s_hist[d * 256 + ((k >> sh.s[d]) & 255u)], 1u);
+__global__ void __launch_bounds__(kSortThreads)
+tile_hist_kernel(const unsigned long long *__restrict__ in, uint32_t n, int shift,
+                 uint32_t *__restrict__ tile_counts, uint32_t *__restrict__ group_counts) {
+    __shared__ uint32_t s_h[256];
+    const int tid = threadIdx.x;
+    if (tid < 256) s_h[tid] = 0;
+    const uint32_t base = blockIdx.x * kSortTile;
+    unsigned long long k[kSortItems];
+    const bool whole = base + kSortTile <= n;
+    if (whole) {                      // 16-byte loads: the tile starts at a multiple of 4,096 keys
+        const ulonglong2 *in2 = reinterpret_cast<const ulonglong2 *>(in + base);
+#pragma unroll
+        for (int it = 0; it < kSortItems / 2; ++it) {
+            const ulonglong2 v = __ldg(in2 + it * kSortThreads + tid);
+            k[2 * it] = v.x;
+            k[2 * it + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int it = 0; it < kSortItems; ++it) {
+            const uint32_t i = base + it * kSortThreads + tid;
+            k[it] = i < n ? __ldg(in + i) : 0ull;
+        }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < sh.n * 256; i += 256)
-        if (s_hist[i]) atomicAdd(hist + i, s_hist[i]);
+#pragma unroll
+    for (int it = 0; it < kSortItems; ++it)
+        if (whole || base + it * kSortThreads + tid < n) atomicAdd(&s_h[(uint32_t)(k[it] >> shift) & 255u], 1u);
+    __syncthreads();
+    if (tid < 256) {
+        const uint32_t c = s_h[tid];
+        tile_counts[(size_t)blockIdx.x * 256 + tid] = c;
+        if (c) add_digit_count(group_counts, blockIdx.x, tid, c, n);
+    }
 }
 
-void launch_key_histograms(cudaStream_t st, const unsigned long long *keys, uint32_t n,
-                           const int *shifts_host, int nd, uint32_t *hist) {
-    if (n == 0 || nd == 0) return;
-    Shifts sh{};
-    sh.n = nd;
-    for (int d = 0; d < nd && d < 8; ++d) sh.s[d] = shifts_host[d];
-    uint32_t g = (n + 4095) / 4096;
-    if (g > 1024) g = 1024;
-    hist_kernel<<<g, 256, 0, st>>>(keys, n, sh, hist);
+// group_counts[g][d] -> digit start(d) + the keys of digit d in earlier
+// groups.  One block: thread (r, d) takes the r-th quarter of the groups.
+__global__ void __launch_bounds__(1024)
+group_scan_kernel(uint32_t *__restrict__ group_counts, uint32_t groups) {
+    __shared__ uint32_t s_part[4][256];
+    __shared__ uint32_t s_scan[256 / 32];
+    const int tid = threadIdx.x, d = tid & 255, r = tid >> 8, lane = tid & 31;
+    const uint32_t per = (groups + 3) / 4, g0 = min(groups, r * per), g1 = min(groups, g0 + per);
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (uint32_t g = g0; g < g1; ++g) sum += group_counts[(size_t)g * 256 + d];
+    s_part[r][d] = sum;
+    __syncthreads();
+    uint32_t inc = 0, tot = 0;
+    if (r == 0) {                     // digit starts: the scan of the 256 totals
+        tot = s_part[0][d] + s_part[1][d] + s_part[2][d] + s_part[3][d];
+        inc = warp_incl_scan(tot);
+        if (lane == 31) s_scan[d >> 5] = inc;
+    }
+    __syncthreads();
+    if (r == 0) {
+        uint32_t run = inc - tot;
+        for (int w = 0; w < (d >> 5); ++w) run += s_scan[w];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t v = s_part[k][d];
+            s_part[k][d] = run;
+            run += v;
+        }
+    }
+    __syncthreads();
+    uint32_t run = s_part[r][d];
+#pragma unroll 8
+    for (uint32_t g = g0; g < g1; ++g) {
+        const uint32_t v = group_counts[(size_t)g * 256 + d];
+        group_counts[(size_t)g * 256 + d] = run;
+        run += v;
+    }
 }
 
-// ---------------------------------------------------------------------------
-// a3: one pass of an onesweep LSD radix sort (8-bit digit at `shift`).
-// A tile of kSortTile keys is ranked in shared memory (warp-private digit
-// histograms built with match-any, so the pass is stable), its digit counts
-// are published for decoupled look-back across tiles (one look-back per
-// digit), and keys are scattered digit-run by digit-run from shared memory so
-// that consecutive threads write consecutive addresses.
-// Status layout: status[digit * num_tiles + tile].
-// ---------------------------------------------------------------------------
-template <bool FINAL, bool PRE>
-__global__ void __launch_bounds__(kSortThreads, FINAL ? 2 : 3)   // 3 tiles in flight per SM (40 registers);
-                                                                  // 2 for the gathering last pass
-onesweep_kernel(const unsigned long long *__restrict__ in, unsigned long long *__restrict__ out,
-                uint32_t n, int shift, const uint32_t *__restrict__ hist256, uint32_t *status,
-                uint32_t *tile_counter, unsigned long long *err, const float2 *__restrict__ pos,
-                uint32_t *__restrict__ skey, uint32_t *__restrict__ sid, float2 *__restrict__ sxy,
-                const uint32_t *__restrict__ tile_offs) {
+// The lanes of the warp whose digit equals this lane's: one ballot per bit.
+// (match-any takes a turn per distinct digit, about 80 cycles for 32 random
+// ones, and bound the pass; eight ballots and their selects issue in 10.)
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d) {
+    uint32_t m = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool p = (d >> b) & 1u;
+        const uint32_t v = __ballot_sync(0xffffffffu, p);
+        m &= p ? v : ~v;
+    }
+    return m;
+}
+
+// Rank and scatter one tile.  Warps rank their keys in private digit counts
+// (stable: items in order, lanes in order); four warps turn the counts into
+// positions in the tile while eight others add up the tile's output starts;
+// the keys are then put in digit order in shared memory and stored run by
+// run, consecutive threads to consecutive addresses.  Keys past n are all
+// ones: they rank behind every key of the last digit and are not stored.
+template <bool FINAL>
+__global__ void __launch_bounds__(kSortThreads, 3)               // 3 tiles in flight per SM (40 registers)
+sort_pass_kernel(const unsigned long long *__restrict__ in, unsigned long long *__restrict__ out,
+                 uint32_t n, int shift, const uint32_t *__restrict__ tile_counts, const uint32_t *__restrict__ group_counts,
+                 int groups_scanned, unsigned long long *err, const float2 *__restrict__ pos,
+                 uint32_t *__restrict__ skey, uint32_t *__restrict__ sid, float2 *__restrict__ sxy) {
     constexpr int W = kSortThreads / 32;
+    static_assert(kSortThreads >= 384 && W * 256 * 2 == kSortThreads * 16, "warp roles and the 16-byte clear");
     __shared__ unsigned long long s_keys[kSortTile];
-    __shared__ uint16_t s_whist[W][256];   // per-warp digit counts (<= 32 * kSortItems)
-    __shared__ uint32_t s_gbase[256];
-    __shared__ uint32_t s_scan[W + 1];
-    __shared__ uint32_t s_tile;
+    __shared__ __align__(16) uint16_t s_whist[W][256];   // per-warp digit counts, then positions in the tile
+    __shared__ uint32_t s_gbase[256], s_dstart[256];
+    __shared__ uint32_t s_part[4], s_part2[8];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (!PRE && tid == 0) s_tile = atomicAdd(tile_counter, 1u);
-    for (int i = tid; i < W * 256; i += kSortThreads) (&s_whist[0][0])[i] = 0;
-    __syncthreads();
-    const uint32_t tile = PRE ? blockIdx.x : s_tile;
-    const uint32_t num_tiles = (n + kSortTile - 1) / kSortTile;
+    const uint32_t tile = blockIdx.x;
     const uint32_t base = tile * kSortTile;
     const uint32_t wbase = base + warp * 32 * kSortItems;
     const uint32_t lt = lanemask_lt();
 
     unsigned long long k[kSortItems];
-    uint32_t r[kSortItems];
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
-        uint32_t idx = wbase + it * 32 + lane;
-        bool valid = idx < n;
-        k[it] = valid ? in[idx] : ~0ull;
+        const uint32_t idx = wbase + it * 32 + lane;
+        k[it] = idx < n ? in[idx] : ~0ull;
     }
+    reinterpret_cast<uint4 *>(&s_whist[0][0])[tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    uint16_t *wh = s_whist[warp];
+    uint32_t r[kSortItems / 2];                    // ranks in the warp's keys (at most 256), two to a register
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
-        uint32_t idx = wbase + it * 32 + lane;
-        bool valid = idx < n;
-        uint32_t dg = valid ? (uint32_t)(k[it] >> shift) & 255u : 256u;
-        uint32_t peers = __match_any_sync(0xffffffffu, dg);
-        int leader = __ffs(peers) - 1;
-        uint32_t before = 0;
-        if (valid && lane == leader) {
-            before = s_whist[warp][dg];
-            s_whist[warp][dg] = before + __popc(peers);
-        }
-        before = __shfl_sync(0xffffffffu, before, leader);
-        r[it] = before + __popc(peers & lt);
+        const uint32_t dg = (uint32_t)(k[it] >> shift) & 255u;
+        const uint32_t peers = digit_peers(dg);
+        const uint32_t rank = wh[dg] + __popc(peers & lt);
         __syncwarp();
+        if ((peers >> lane) == 1u) wh[dg] = (uint16_t)(rank + 1u);      // the last of its peers
+        __syncwarp();
+        if (it & 1) r[it / 2] |= rank << 16;
+        else r[it / 2] = rank;
     }
     __syncthreads();
 
-    // Per digit (thread tid == digit, tid < 256): exclusive prefix over warps,
-    // tile-local digit starts, output start of the tile's keys of that digit.
-    uint32_t c = 0;
-    if (tid < 256) {
+    if (warp < 4) {
+        // digits 2 tid and 2 tid + 1, packed: the warps' exclusive counts, then the digits' starts
+        uint32_t c = 0;
+        uint32_t *col = reinterpret_cast<uint32_t *>(&s_whist[0][0]) + tid;
 #pragma unroll
+        for (int w = 0; w < W; ++w) c += col[w * 128];
+        const uint32_t c0 = c & 0xffffu, c1 = c >> 16;
+        const uint32_t inc = warp_incl_scan(c0 + c1);
+        if (lane == 31) s_part[warp] = inc;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        uint32_t d0 = inc - c0 - c1;
+        for (int w = 0; w < warp; ++w) d0 += s_part[w];
+        s_dstart[2 * tid] = d0;
+        s_dstart[2 * tid + 1] = d0 + c0;
+        uint32_t run = d0 | ((d0 + c0) << 16);         // positions are below 4,096: no carry between the halves
+#pragma unroll 4
         for (int w = 0; w < W; ++w) {
-            uint32_t v = s_whist[w][tid];
-            s_whist[w][tid] = c;
-            c += v;
+            const uint32_t v = col[w * 128];
+            col[w * 128] = run;
+            run += v;
         }
-    }
-    uint32_t tot;
-    uint32_t dstart = block_excl_scan<kSortThreads>(c, &tot, s_scan);
-    // each warp's slot for its first key of digit tid: the digit's start in
-    // the tile plus the warp's exclusive count (one table read per key below)
-    if (tid < 256) {
-#pragma unroll 1
-        for (int w = 0; w < W; ++w) s_whist[w][tid] = (uint16_t)(s_whist[w][tid] + dstart);
-    }
-    if (PRE) {
-        // output start of this tile's keys of digit tid, from the tile-histogram scan
-        if (tid < 256) s_gbase[tid] = tile_offs[(size_t)tid * num_tiles + tile] - dstart;
-    } else {
-        uint32_t gstart = block_excl_scan<kSortThreads>(tid < 256 ? hist256[tid] : 0u, &tot, s_scan);
-        if (tid < 256) {
-            uint32_t prefix = lookback1<uint32_t>(status + (size_t)tid * num_tiles, tile, c, err);
-            s_gbase[tid] = gstart + prefix - dstart;
+    } else if (warp < 12) {
+        const uint32_t d = tid - 128, g = tile / kSortGroup;
+        uint32_t start = 0;
+        if (groups_scanned) {
+            start = __ldg(group_counts + (size_t)(kSortTotalRows + g) * 256 + d);
+        } else {
+            uint32_t total = 0, before = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < kSortTotalRows; ++j) total += __ldg(group_counts + (size_t)j * 256 + d);
+#pragma unroll 8
+            for (uint32_t j = 0; j < g; ++j) before += __ldg(group_counts + (size_t)(kSortTotalRows + j) * 256 + d);
+            const uint32_t inc = warp_incl_scan(total);
+            if (lane == 31) s_part2[d >> 5] = inc;
+            asm volatile("bar.sync 2, 256;" ::: "memory");
+            start = inc - total + before;
+            for (uint32_t w = 0; w < (d >> 5); ++w) start += s_part2[w];
         }
+#pragma unroll 8
+        for (uint32_t t = g * kSortGroup; t < tile; ++t) start += __ldg(tile_counts + (size_t)t * 256 + d);
+        s_gbase[d] = start;
     }
     __syncthreads();
 
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
-        uint32_t idx = wbase + it * 32 + lane;
-        if (idx < n) {
-            uint32_t dg = (uint32_t)(k[it] >> shift) & 255u;
-            s_keys[s_whist[warp][dg] + r[it]] = k[it];
-        }
+        const uint32_t dg = (uint32_t)(k[it] >> shift) & 255u;
+        s_keys[wh[dg] + ((it & 1) ? r[it / 2] >> 16 : r[it / 2] & 0xffffu)] = k[it];
     }
+    if (tid < 256) s_gbase[tid] -= s_dstart[tid];
     __syncthreads();
 
     const uint32_t nvalid = n - base < (uint32_t)kSortTile ? n - base : (uint32_t)kSortTile;
-    if (FINAL) {
-        // The last pass gathers each object's position by id (random reads):
-        // all of a thread's gathers are issued before any store so they overlap.
-        float2 pv[kSortItems];
-        unsigned long long kv[kSortItems];
-        uint32_t ov[kSortItems];
+    if constexpr (FINAL) {
+        // The last pass splits keys and ids and, unless sxy is null, gathers
+        // each object's position by id (random reads),
+        // four gathers of a thread in flight.  (Eight at 64 registers, two
+        // tiles per SM: 49 us against 45 at 4M objects, 116 against 103 at 12M.)
+#pragma unroll 1
+        for (int b = 0; b < kSortItems; b += 4) {
+            float2 pv[4];
 #pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            const uint32_t i = tid + j * kSortThreads;
-            ov[j] = n;                                  // n: nothing to write
-            if (i < nvalid) {
-                kv[j] = s_keys[i];
-                ov[j] = s_gbase[(uint32_t)(kv[j] >> shift) & 255u] + i;
-                const uint32_t kk = (uint32_t)(kv[j] >> 32);
-                if (ov[j] < n && kk != kAbsentKey) pv[j] = pos[(uint32_t)kv[j]];
-                if (ov[j] >= n) atomicOr(err, kErrInternal);
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t i = tid + (b + j) * kSortThreads;
+                if (i < nvalid) {
+                    const unsigned long long key = s_keys[i];
+                    if (sxy && (uint32_t)(key >> 32) != kAbsentKey) pv[j] = pos[(uint32_t)key];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t i = tid + (b + j) * kSortThreads;
+                if (i >= nvalid) continue;
+                const unsigned long long key = s_keys[i];
+                const uint32_t o = s_gbase[(uint32_t)(key >> shift) & 255u] + i;
+                if (o >= n) {
+                    atomicOr(err, kErrInternal);
+                    continue;
+                }
+                skey[o] = (uint32_t)(key >> 32);
+                sid[o] = (uint32_t)key;
+                if (sxy && (uint32_t)(key >> 32) != kAbsentKey) sxy[o] = pv[j];
             }
         }
+    } else {
+        for (uint32_t i = tid; i < nvalid; i += kSortThreads) {
+            const unsigned long long key = s_keys[i];
+            const uint32_t o = s_gbase[(uint32_t)(key >> shift) & 255u] + i;
+            if (o >= n) {
+                atomicOr(err, kErrInternal);
+                continue;
+            }
+            out[o] = key;
+        }
+    }
+}
+
+void launch_sort_pass(cudaStream_t st, const unsigned long long *in, unsigned long long *out, uint32_t n,
+                      int shift, uint32_t *tile_counts, uint32_t *group_counts, bool counts_ready,
+                      unsigned long long *err, bool final_obj, const float2 *pos, uint32_t *skey, uint32_t *sid,
+                      float2 *sxy) {
+    if (n == 0) return;
+    const uint32_t tiles = sort_tiles(n), groups = sort_groups(n);
+    if (!counts_ready) tile_hist_kernel<<<tiles, kSortThreads, 0, st>>>(in, n, shift, tile_counts, group_counts);
+    const int scanned = groups > kSortDirectGroups ? 1 : 0;
+    if (scanned) group_scan_kernel<<<1, 1024, 0, st>>>(group_counts + (size_t)kSortTotalRows * 256, groups);
+    if (final_obj)
+        sort_pass_kernel<true><<<tiles, kSortThreads, 0, st>>>(in, out, n, shift, tile_counts, group_counts, scanned,
+                                                              err, pos, skey, sid, sxy);
+    else
+        sort_pass_kernel<false><<<tiles, kSortThreads, 0, st>>>(in, out, n, shift, tile_counts, group_counts, scanned,
+                                                               err, nullptr, nullptr, nullptr, nullptr);
+}
+
+uint32_t sort_pass_launches(uint32_t n, bool counts_ready) {
+    if (n == 0) return 0;
+    return 1u + (counts_ready ? 0u : 1u) + (sort_groups(n) > kSortDirectGroups ? 1u : 0u);
+}
+
+// ---------------------------------------------------------------------------
+// a2 + a3 for small populations: keys and all four sort passes in one launch,
+// by one thread-block cluster.  The keys never leave the SMs: every block
+// ranks its keys in shared memory, the blocks read each other's 256 digit
+// totals, and each key is stored into the shared memory of the block that
+// holds its new position (two cluster barriers per pass).  Launches, barriers
+// and latency bound a sort of this size.  Keys and sort, by events: 58 us ->
+// 21 at 4,096 objects, 62 -> 27 at 16,384, 69 -> 46 at 65,536; at 131,072 the
+// passes of a launch each (71 us) are faster than this kernel (75).
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 1024, kSmallWarps = kSmallThreads / 32;
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
+    return a;
+}
+
+// The grid is one cluster; block r holds the positions [r * T, (r + 1) * T),
+// T = 1024 * ITEMS.  stamp may be null (every object is present), sxy and
+// info too (keys and ids only).
+template <int ITEMS>
+__global__ void __launch_bounds__(kSmallThreads, 1)
+small_sort_kernel(const float2 *__restrict__ pos, const unsigned long long *__restrict__ stamp, uint32_t n,
+                  float x0, float y0, float sx, float sy, Worlds worlds, uint32_t *__restrict__ skey,
+                  uint32_t *__restrict__ sid, float2 *__restrict__ sxy, Info *info) {
+    constexpr uint32_t T = kSmallThreads * ITEMS;
+    extern __shared__ unsigned long long s_keys[];              // T keys
+    __shared__ __align__(16) uint16_t s_whist[kSmallWarps][256];
+    __shared__ uint32_t s_seg[8][128];                          // digit pairs: counts of eight groups of four warps
+    __shared__ uint32_t s_tot[256], s_base[256], s_part[8], s_cnt;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t rank = cluster_rank(), nblocks = gridDim.x;
+    const uint32_t p0 = rank * T + warp * 32 * ITEMS + lane;
+    const uint32_t lt = lanemask_lt();
+    const uint32_t keys_addr = (uint32_t)__cvta_generic_to_shared(s_keys);
+    const uint32_t tot_addr = (uint32_t)__cvta_generic_to_shared(s_tot);
+    if (tid == 0) s_cnt = 0;
+
+    unsigned long long k[ITEMS];
+    uint32_t present = 0;
 #pragma unroll
-        for (int j = 0; j < kSortItems; ++j) {
-            if (ov[j] >= n) continue;
-            const uint32_t kk = (uint32_t)(kv[j] >> 32);
-            skey[ov[j]] = kk;
-            sid[ov[j]] = (uint32_t)kv[j];
-            if (kk != kAbsentKey) sxy[ov[j]] = pv[j];
+    for (int it = 0; it < ITEMS; ++it) {
+        const uint32_t i = p0 + it * 32;
+        k[it] = ~0ull;
+        if (i < n) {
+            uint32_t key = kAbsentKey;
+            if (!stamp || stamp[i] != 0ull) {
+                const float2 p = pos[i];
+                uint32_t ci = cell_of(p.x, x0, sx), cj = cell_of(p.y, y0, sy);
+                if (worlds.n) {
+                    const uint32_t w = world_of(i, worlds.obj_base, 0, worlds.n);
+                    ci = world_cell(ci, w, worlds.bits, 0);
+                    cj = world_cell(cj, w, worlds.bits, 1);
+                }
+                key = morton2(ci, cj);
+                ++present;
+            }
+            k[it] = ((unsigned long long)key << 32) | i;
         }
-        return;
     }
-    for (uint32_t i = tid; i < nvalid; i += kSortThreads) {
-        unsigned long long key = s_keys[i];
-        uint32_t dg = (uint32_t)(key >> shift) & 255u;
-        uint32_t o = s_gbase[dg] + i;
-        if (o >= n) {
-            atomicOr(err, kErrInternal);
-            continue;
-        }
-        out[o] = key;
-    }
-}
-
-void launch_onesweep_pass(cudaStream_t st, const unsigned long long *in, unsigned long long *out,
-                          uint32_t n, int shift, const uint32_t *hist256, uint32_t *status,
-                          uint32_t *tile_counter, unsigned long long *err, bool final_obj,
-                          const float2 *pos, uint32_t *skey, uint32_t *sid, float2 *sxy) {
-    if (n == 0) return;
-    uint32_t tiles = (n + kSortTile - 1) / kSortTile;
-    if (final_obj)
-        onesweep_kernel<true, false><<<tiles, kSortThreads, 0, st>>>(in, out, n, shift, hist256, status,
-                                                                    tile_counter, err, pos, skey, sid, sxy,
-                                                                    nullptr);
-    else
-        onesweep_kernel<false, false><<<tiles, kSortThreads, 0, st>>>(in, out, n, shift, hist256, status,
-                                                                     tile_counter, err, pos, skey, sid, sxy,
-                                                                     nullptr);
-}
-
-// ---------------------------------------------------------------------------
-// a3, look-back-free pass (when every tile of a pass runs in one wave the
-// decoupled look-back degenerates into a serial walk): per-tile digit counts,
-// then one block per digit scans its counts over the tiles (adding the
-// digit's global start), then the same stable rank-and-scatter tile kernel
-// reads its offsets instead of looking back.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads)
-tile_hist_kernel(const unsigned long long *__restrict__ in, uint32_t n, int shift,
-                 uint32_t *__restrict__ counts) {
-    __shared__ uint32_t s_h[256];
-    const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
-    for (int i = threadIdx.x; i < 256; i += kSortThreads) s_h[i] = 0;
     __syncthreads();
-    const uint32_t base = blockIdx.x * kSortTile;
+    if (info) {
+        present = warp_sum(present);
+        if (lane == 0 && present) atomicAdd(&s_cnt, present);
+    }
+#pragma unroll 1
+    for (int shift = 32; shift < 64; shift += 8) {
+        if (shift > 32) {
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) k[it] = s_keys[warp * 32 * ITEMS + it * 32 + lane];
+        }
+        reinterpret_cast<uint4 *>(&s_whist[0][0])[tid] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        uint16_t *wh = s_whist[warp];
+        uint32_t r[(ITEMS + 1) / 2];                            // ranks in the warp's keys (at most 512)
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const uint32_t dg = (uint32_t)(k[it] >> shift) & 255u;
+            const uint32_t peers = digit_peers(dg);
+            const uint32_t rk = wh[dg] + __popc(peers & lt);
+            __syncwarp();
+            if ((peers >> lane) == 1u) wh[dg] = (uint16_t)(rk + 1u);
+            __syncwarp();
+            if (it & 1) r[it / 2] |= rk << 16;
+            else r[it / 2] = rk;
+        }
+        __syncthreads();
+        // the warps' counts to the block's exclusive counts, two digits to a
+        // word: thread (g, c) takes digit pair c of four warps
+        {
+            const int g = tid >> 7, c = tid & 127;
+            uint32_t *col = reinterpret_cast<uint32_t *>(&s_whist[0][0]) + g * 4 * 128 + c;
+            uint32_t v[4], sum = 0;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                v[w] = col[w * 128];
+                sum += v[w];
+            }
+            s_seg[g][c] = sum;
+            __syncthreads();
+            uint32_t run = 0, tot = 0;
+#pragma unroll
+            for (int h = 0; h < 8; ++h) {
+                const uint32_t x = s_seg[h][c];
+                if (h < g) run += x;
+                tot += x;
+            }
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                col[w * 128] = run;
+                run += v[w];
+            }
+            if (g == 0) {
+                s_tot[2 * c] = tot & 0xffffu;
+                s_tot[2 * c + 1] = tot >> 16;
+            }
+        }
+        cluster_barrier();                                      // every block's totals are out, its keys read
+        uint32_t before = 0, all = 0, inc = 0;
+        if (tid < 256) {
+            for (uint32_t q = 0; q < nblocks; ++q) {
+                uint32_t v;
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_map(tot_addr, q) + 4u * tid));
+                if (q < rank) before += v;
+                all += v;
+            }
+            inc = warp_incl_scan(all);
+            if (lane == 31) s_part[warp] = inc;
+        }
+        __syncthreads();
+        if (tid < 256) {
+            uint32_t start = inc - all + before;
+            for (int w = 0; w < warp; ++w) start += s_part[w];
+            s_base[tid] = start;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const uint32_t dg = (uint32_t)(k[it] >> shift) & 255u;
+            const uint32_t o = s_base[dg] + wh[dg] + ((it & 1) ? r[it / 2] >> 16 : r[it / 2] & 0xffffu);
+            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_map(keys_addr, o / T) + 8u * (o % T)),
+                         "l"(k[it]) : "memory");
+        }
+        cluster_barrier();                                      // the keys have arrived
+    }
+    if (info && tid == 0 && s_cnt) atomicAdd(&info->n_present, (unsigned long long)s_cnt);
 #pragma unroll 4
-    for (int it = 0; it < kSortItems; ++it) {
-        const uint32_t i = base + it * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&s_h[(uint32_t)(in[i] >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += kSortThreads) counts[(size_t)i * tiles + blockIdx.x] = s_h[i];
-}
-
-__global__ void __launch_bounds__(256)
-digit_scan_kernel(const uint32_t *__restrict__ counts, const uint32_t *__restrict__ hist256, uint32_t n,
-                  uint32_t *__restrict__ offs) {
-    __shared__ uint32_t s_scan[256 / 32 + 1];
-    __shared__ uint32_t s_base;
-    const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
-    const uint32_t d = blockIdx.x;
-    uint32_t tot;
-    const uint32_t g = block_excl_scan<256>(hist256[threadIdx.x], &tot, s_scan);
-    if (threadIdx.x == d) s_base = g;
-    __syncthreads();
-    uint32_t carry = s_base;
-    const uint32_t *cd = counts + (size_t)d * tiles;
-    uint32_t *od = offs + (size_t)d * tiles;
-    for (uint32_t t0 = 0; t0 < tiles; t0 += 256) {
-        const uint32_t t = t0 + threadIdx.x;
-        const uint32_t v = t < tiles ? cd[t] : 0u;
-        uint32_t chunk;
-        const uint32_t ex = block_excl_scan<256>(v, &chunk, s_scan);
-        if (t < tiles) od[t] = carry + ex;
-        carry += chunk;
+    for (uint32_t j = tid; j < T; j += kSmallThreads) {
+        const uint32_t o = rank * T + j;
+        if (o >= n) break;
+        const unsigned long long key = s_keys[j];
+        skey[o] = (uint32_t)(key >> 32);
+        sid[o] = (uint32_t)key;
+        if (sxy && (uint32_t)(key >> 32) != kAbsentKey) sxy[o] = pos[(uint32_t)key];
     }
 }
 
-void launch_sort_pass_pre(cudaStream_t st, const unsigned long long *in, unsigned long long *out, uint32_t n,
-                          int shift, const uint32_t *hist256, uint32_t *counts, uint32_t *offs,
-                          unsigned long long *err, bool final_obj, const float2 *pos, uint32_t *skey,
-                          uint32_t *sid, float2 *sxy, bool counts_ready) {
-    if (n == 0) return;
-    const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
-    if (!counts_ready) tile_hist_kernel<<<tiles, kSortThreads, 0, st>>>(in, n, shift, counts);
-    digit_scan_kernel<<<256, 256, 0, st>>>(counts, hist256, n, offs);
-    if (final_obj)
-        onesweep_kernel<true, true><<<tiles, kSortThreads, 0, st>>>(in, out, n, shift, hist256, nullptr,
-                                                                   nullptr, err, pos, skey, sid, sxy, offs);
-    else
-        onesweep_kernel<false, true><<<tiles, kSortThreads, 0, st>>>(in, out, n, shift, hist256, nullptr,
-                                                                    nullptr, err, pos, skey, sid, sxy, offs);
+// A cluster of at most 16 blocks (twice the portable size: at 32,768 objects
+// 33 us against 42 with eight blocks of twice the keys).
+constexpr uint32_t kSmallBlocks = 16;
+static_assert(kSmallSortMax == kSmallBlocks * kSmallThreads * 4, "four items at most");
+
+template <int ITEMS>
+static cudaLaunchConfig_t small_config(uint32_t n, cudaStream_t st, cudaLaunchAttribute *attr) {
+    constexpr uint32_t T = kSmallThreads * ITEMS;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (n + T - 1) / T;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((n + T - 1) / T);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = T * sizeof(unsigned long long);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <int ITEMS>
+static bool small_ready_items() {
+    if (cudaFuncSetAttribute(small_sort_kernel<ITEMS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        return false;
+    cudaLaunchAttribute attr{};
+    const cudaLaunchConfig_t cfg = small_config<ITEMS>(kSmallBlocks * kSmallThreads * ITEMS, nullptr, &attr);
+    int clusters = 0;
+    return cudaOccupancyMaxActiveClusters(&clusters, small_sort_kernel<ITEMS>, &cfg) == cudaSuccess && clusters > 0;
+}
+
+bool small_sort_ready() {
+    static_assert(kSmallThreads * 4 * sizeof(unsigned long long) + sizeof(uint16_t) * kSmallWarps * 256 + 8192 <=
+                      57344, "dynamic and static shared memory");
+    const bool ok = cudaFuncSetAttribute(small_sort_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kSmallThreads * 4 * sizeof(unsigned long long))) == cudaSuccess &&
+                    small_ready_items<1>() && small_ready_items<2>() && small_ready_items<4>();
+    if (!ok) (void)cudaGetLastError();
+    return ok;
+}
+
+template <int ITEMS>
+static cudaError_t launch_small_items(cudaStream_t st, const float2 *pos, const unsigned long long *stamp, uint32_t n,
+                                      float x0, float y0, float sx, float sy, Worlds worlds, uint32_t *skey,
+                                      uint32_t *sid, float2 *sxy, Info *info) {
+    cudaLaunchAttribute attr{};
+    const cudaLaunchConfig_t cfg = small_config<ITEMS>(n, st, &attr);
+    return cudaLaunchKernelEx(&cfg, small_sort_kernel<ITEMS>, pos, stamp, n, x0, y0, sx, sy, worlds, skey, sid, sxy,
+                              info);
+}
+
+cudaError_t launch_small_sort(cudaStream_t st, const float2 *pos, const unsigned long long *stamp, uint32_t n,
+                              float x0, float y0, float sx, float sy, Worlds worlds, uint32_t *skey, uint32_t *sid,
+                              float2 *sxy, Info *info) {
+    if (n == 0) return cudaSuccess;
+    if (n <= kSmallBlocks * kSmallThreads)
+        return launch_small_items<1>(st, pos, stamp, n, x0, y0, sx, sy, worlds, skey, sid, sxy, info);
+    if (n <= kSmallBlocks * kSmallThreads * 2)
+        return launch_small_items<2>(st, pos, stamp, n, x0, y0, sx, sy, worlds, skey, sid, sxy, info);
+    return launch_small_items<4>(st, pos, stamp, n, x0, y0, sx, sy, worlds, skey, sid, sxy, info);
 }
 
 // ---------------------------------------------------------------------------

@@ -145,7 +145,7 @@ query_blocks_kernel(const float4 *__restrict__ rects, uint32_t Q, float x0, floa
     QCells c;
     const bool qok = qvalid && L > 0 && query_cells(rects[q], x0, y0, sx, sy, c);
     if (qok && worlds.n) {      // the query's cells inside its world's node
-        const uint32_t w = world_of(q, worlds.q_base, worlds.n);
+        const uint32_t w = world_of(q, worlds.q_base, 0, worlds.n);
         c.i0 = world_cell(c.i0, w, worlds.bits, 0);
         c.i1 = world_cell(c.i1, w, worlds.bits, 0);
         c.j0 = world_cell(c.j0, w, worlds.bits, 1);

@@ -1,6 +1,6 @@
 // mqr_api.cu -- the C ABI of libmqr (declared in include/mqr.h): context,
 // device memory, and the per-tick pipeline
-//   a2 Morton keys -> a3 onesweep sort (4 passes) -> a4 leaves ->
+//   a2 Morton keys -> a3 radix sort (4 passes) -> a4 leaves ->
 //   a5/a6 query count + scan -> a8 leaf scans -> a7 query write ->
 //   a10 filter -> a11 result scan -> a12/a13 emit (-> a14 sort/layout)
 // all enqueued on the context's stream with one host synchronisation at the
@@ -90,6 +90,7 @@ struct mqr_ctx {
     mqr_rect bounds{};
     float sx = 0.f, sy = 0.f;
     uint32_t nmax = 0;
+    bool small_sort = false;        // keys and sort in one launch
     unsigned long long epoch = 0;
 
     // resident state
@@ -97,7 +98,7 @@ struct mqr_ctx {
     DevBuf<unsigned long long> stamp;
     // sort
     DevBuf<unsigned long long> keysA, keysB;
-    DevBuf<uint32_t> skey, sid, sort_counts, sort_offs;
+    DevBuf<uint32_t> skey, sid, sort_counts;
     DevBuf<float2> sxy;
     // leaves
     DevBuf<uint32_t> leaf_lo, leaf_hi, leaf_beg, leaf_nsub, leaf_sub_off, leaf_word_off,
@@ -112,7 +113,7 @@ struct mqr_ctx {
     DevBuf<uint2> qcells;
     DevBuf<unsigned long long> cand_off, pair_off;
     unsigned long long cand_tiles = 0;
-    // zero-initialised arena: Info, histograms, tile counters, look-back status
+    // zero-initialised arena: Info, tile counters, coarse digit counts, look-back status
     DevBuf<unsigned char> arena;
     // staging for the host-buffer entry points and the sorted output kinds
     DevBuf<uint32_t> up_ids;
@@ -223,19 +224,15 @@ struct mqr_ctx {
 
 namespace {
 
-// The object sort runs its passes with look-back up to this many tiles.
-constexpr uint32_t kSortLookbackTiles = 16;
-
 // Arena layout for one tick.
 struct Arena {
-    size_t info, hist, counters, st_sort, st_leaf, st_lscan, st_qb_p, st_qb_c, st_cand, st_res, total;
-    uint32_t sort_tiles, leaf_tiles, lscan_tiles, qb_tiles, res_tiles;
+    size_t info, counters, sort_group, st_leaf, st_lscan, st_qb_p, st_qb_c, st_cand, st_res, total;
+    uint32_t leaf_tiles, lscan_tiles, qb_tiles, res_tiles;
     unsigned long long cand_tiles;
 };
 
 Arena arena_layout(uint32_t nmax, uint32_t Q, unsigned long long sub_cap, unsigned long long cand_tiles) {
     Arena a{};
-    a.sort_tiles = (nmax + kSortTile - 1) / kSortTile;
     a.leaf_tiles = (nmax + kLeafTile - 1) / kLeafTile;
     a.lscan_tiles = (nmax + kLeafScanTile - 1) / kLeafScanTile;
     a.qb_tiles = (Q + kQBQueries - 1) / kQBQueries;
@@ -248,11 +245,8 @@ Arena arena_layout(uint32_t nmax, uint32_t Q, unsigned long long sub_cap, unsign
         return r;
     };
     a.info = take(sizeof(Info));
-    a.hist = take(8 * 256 * sizeof(uint32_t));
     a.counters = take(16 * sizeof(uint32_t));
-    // look-back status of the object sort's four passes, when it runs them
-    // with look-back (a few tiles: see enqueue_index)
-    a.st_sort = take(a.sort_tiles <= kSortLookbackTiles ? (size_t)4 * 256 * a.sort_tiles * sizeof(uint32_t) : 0);
+    a.sort_group = take(4 * sort_group_words(nmax) * sizeof(uint32_t));   // a set per pass
     a.st_leaf = take((size_t)a.leaf_tiles * sizeof(uint32_t));
     a.st_lscan = take((size_t)3 * a.lscan_tiles * sizeof(uint32_t));
     a.st_qb_p = take((size_t)a.qb_tiles * sizeof(uint32_t));
@@ -381,51 +375,46 @@ mqr_status wait_for_slots(mqr_ctx *c) {
     return MQR_OK;
 }
 
-// a2 - a4: Morton keys, the onesweep sort and the leaves of the current
+// a2 - a4: Morton keys, the radix sort and the leaves of the current
 // state, then the snapshot's counters for the slots.  The arena is zeroed and
 // the update kernels' error bits carried in first.
 mqr_status enqueue_index(mqr_ctx *c, const Arena &a) {
     cudaStream_t st = c->stream;
     Info *info = at<Info>(c, a.info);
-    uint32_t *hist = at<uint32_t>(c, a.hist);
     uint32_t *ctr = at<uint32_t>(c, a.counters);
     unsigned long long *err = &info->err;
     const float x0 = c->bounds.xmin, y0 = c->bounds.ymin;
     const uint32_t nmax = c->nmax;
     mqr_status s = wait_for_slots(c);
     if (s != MQR_OK) return s;
-    MQR_CUDA(cudaMemsetAsync(c->arena.p, 0, a.total, st));
-    // Carry the update kernels' sticky error bits into this tick.
-    MQR_CUDA(cudaMemcpyAsync(&info->err, c->upd_err.p, sizeof(unsigned long long),
-                             cudaMemcpyDeviceToDevice, st));
-    MQR_CUDA(cudaMemsetAsync(c->upd_err.p, 0, sizeof(unsigned long long), st));
-
-    // a2 + a3: keys and the 4-pass onesweep sort of (key << 32 | id).
+    // a2 + a3: the counters cleared and the update kernels' sticky error bits
+    // carried into this tick, then keys and the 4-pass radix sort of (key << 32 | id).
     phase_begin(c, MQR_PHASE_KEYS);
+    launch_tick_begin(st, c->arena.p, a.total, c->upd_err.p, nullptr);
     const Worlds worlds{c->world_obj.p, c->world_q.p, c->n_worlds, c->world_bits};
-    launch_morton_keys(st, c->pos.p, c->stamp.p, nmax, x0, y0, c->sx, c->sy, worlds, c->keysA.p, hist,
-                       c->sort_counts.p, info);
-    phase_end(c, MQR_PHASE_KEYS, nmax ? 1 : 0);
-    unsigned long long *src = c->keysA.p, *dst = c->keysB.p;
-    phase_begin(c, MQR_PHASE_SORT);
-    // A few tiles: each pass's tiles look back over one another (one launch
-    // per pass; the walk is short); more: the look-back-free passes (tile
-    // counts, digit scan, rank and scatter), whose tiles need not wait.
-    const bool sort_lookback = a.sort_tiles <= kSortLookbackTiles;
-    uint32_t *st_sort = at<uint32_t>(c, a.st_sort);
-    for (int p = 0; p < 4; ++p) {
-        const bool fin = p == 3;
-        if (sort_lookback)
-            launch_onesweep_pass(st, src, dst, nmax, 32 + 8 * p, hist + 256 * p,
-                                 st_sort + (size_t)256 * a.sort_tiles * p, ctr + p, err, fin, c->pos.p, c->skey.p,
-                                 c->sid.p, c->sxy.p);
-        else
-            launch_sort_pass_pre(st, src, dst, nmax, 32 + 8 * p, hist + 256 * p, c->sort_counts.p,
-                                 c->sort_offs.p, err, fin, c->pos.p, c->skey.p, c->sid.p, c->sxy.p, p == 0);
-        std::swap(src, dst);
+    if (c->small_sort) {                        // one launch for the keys and the sort (timed as the sort)
+        phase_end(c, MQR_PHASE_KEYS, 1);
+        phase_begin(c, MQR_PHASE_SORT);
+        MQR_CUDA(launch_small_sort(st, c->pos.p, c->stamp.p, nmax, x0, y0, c->sx, c->sy, worlds, c->skey.p, c->sid.p,
+                                   c->sxy.p, info));
+        phase_end(c, MQR_PHASE_SORT, nmax ? 1 : 0);
+    } else {
+        uint32_t *groups = at<uint32_t>(c, a.sort_group);
+        const size_t group_words = sort_group_words(nmax);
+        launch_morton_keys(st, c->pos.p, c->stamp.p, nmax, x0, y0, c->sx, c->sy, worlds, c->keysA.p,
+                           c->sort_counts.p, groups, info);
+        phase_end(c, MQR_PHASE_KEYS, 2);
+        unsigned long long *src = c->keysA.p, *dst = c->keysB.p;
+        phase_begin(c, MQR_PHASE_SORT);
+        uint64_t sort_launches = 0;
+        for (int p = 0; p < 4; ++p) {              // the first pass's digit counts come from the key kernel
+            launch_sort_pass(st, src, dst, nmax, 32 + 8 * p, c->sort_counts.p, groups + group_words * p, p == 0, err,
+                             p == 3, c->pos.p, c->skey.p, c->sid.p, c->sxy.p);
+            sort_launches += sort_pass_launches(nmax, p == 0);
+            std::swap(src, dst);
+        }
+        phase_end(c, MQR_PHASE_SORT, sort_launches);
     }
-    // the look-back-free passes: the first pass's tile counts come from the key kernel
-    phase_end(c, MQR_PHASE_SORT, nmax ? (sort_lookback ? 4 : 11) : 0);
     // a4
     phase_begin(c, MQR_PHASE_LEAVES);
     const uint32_t cap = c->cfg.leaf_cap;
@@ -463,8 +452,8 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
                         bool admit) {
     cudaStream_t st = c->stream;
     Info *info = at<Info>(c, a.info);
-    // tile/ticket counters: 0-3 sort passes, 4 leaves, 5 query blocks, 6 leaf scan, 7 result scan,
-    // 8 candidate scan, 9 emit batches, 10 filter items; 12-13 the output sort's error word
+    // tile/ticket counters: 4 leaves, 5 query blocks, 6 leaf scan, 7 result scan,
+    // 8 candidate scan, 9 emit batches, 10 filter items
     uint32_t *ctr = at<uint32_t>(c, a.counters);
     const float x0 = c->bounds.xmin, y0 = c->bounds.ymin;
     const uint32_t nmax = c->nmax;
@@ -561,13 +550,8 @@ mqr_status enqueue_tick(mqr_ctx *c, const float4 *rects, uint32_t Q, int emit_ki
 mqr_status enqueue_slot(mqr_ctx *c, const float4 *rects, uint32_t Q, int emit_kind, void *out,
                         unsigned long long out_cap_elems, unsigned long long *offsets, const Arena &a, Caps &caps) {
     const mqr_ctx *ix = c->parent;
-    Info *info = at<Info>(c, a.info);
-    MQR_CUDA(cudaMemsetAsync(c->arena.p, 0, a.total, c->stream));
     MQR_CUDA(cudaStreamWaitEvent(c->stream, ix->snap_ready, 0));
-    MQR_CUDA(cudaMemcpyAsync(info, ix->snap_info.p, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice,
-                             c->stream));
-    MQR_CUDA(cudaMemcpyAsync(&info->err, ix->snap_info.p + 3, sizeof(unsigned long long), cudaMemcpyDeviceToDevice,
-                             c->stream));
+    launch_tick_begin(c->stream, c->arena.p, a.total, nullptr, ix->snap_info.p);
     return enqueue_join(c, ix, rects, Q, emit_kind, out, out_cap_elems, offsets, a, caps, true);
 }
 
@@ -778,23 +762,19 @@ mqr_status sort_result_keys(mqr_ctx *c, uint64_t n, uint32_t Q, unsigned long lo
     while (qbits < 32 && (1ull << qbits) < Q) ++qbits;
     for (uint32_t b = 0; b < idbits; b += 8) shifts[nd++] = (int)b;
     for (uint32_t b = 0; b < qbits; b += 8) shifts[nd++] = 32 + (int)b;
-    uint32_t tiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
-    size_t hist_off = 0, ctr_off = 8 * 256 * sizeof(uint32_t);
-    size_t st_off = ctr_off + 256;
-    size_t total = st_off + (size_t)nd * 256 * tiles * sizeof(uint32_t);
-    MQR_CUDA(c->sort_arena.ensure(total));
-    MQR_CUDA(cudaMemsetAsync(c->sort_arena.p, 0, total, c->stream));
-    uint32_t *hist = reinterpret_cast<uint32_t *>(c->sort_arena.p + hist_off);
-    uint32_t *ctr = reinterpret_cast<uint32_t *>(c->sort_arena.p + ctr_off);
-    uint32_t *stp = reinterpret_cast<uint32_t *>(c->sort_arena.p + st_off);
-    launch_key_histograms(c->stream, c->sortA.p, (uint32_t)n, shifts, nd, hist);
+    const size_t tile_words = (size_t)256 * sort_tiles((uint32_t)n), group_words = sort_group_words((uint32_t)n);
+    const size_t group_off = 256;
+    const size_t tile_off = group_off + (size_t)nd * group_words * sizeof(uint32_t);
+    MQR_CUDA(c->sort_arena.ensure(tile_off + tile_words * sizeof(uint32_t)));
+    MQR_CUDA(cudaMemsetAsync(c->sort_arena.p, 0, tile_off, c->stream));
+    // error word of this sort
+    unsigned long long *err = reinterpret_cast<unsigned long long *>(c->sort_arena.p);
+    uint32_t *group = reinterpret_cast<uint32_t *>(c->sort_arena.p + group_off);
+    uint32_t *tile = reinterpret_cast<uint32_t *>(c->sort_arena.p + tile_off);
     unsigned long long *src = c->sortA.p, *dst = c->sortB.p;
-    // error word of this sort: a dedicated slot in its counters block
-    unsigned long long *err = reinterpret_cast<unsigned long long *>(ctr + 12);
     for (int d = 0; d < nd; ++d) {
-        launch_onesweep_pass(c->stream, src, dst, (uint32_t)n, shifts[d], hist + 256 * d,
-                             stp + (size_t)256 * tiles * d, ctr + d, err, false, nullptr, nullptr,
-                             nullptr, nullptr);
+        launch_sort_pass(c->stream, src, dst, (uint32_t)n, shifts[d], tile, group + group_words * d, false, err,
+                         false, nullptr, nullptr, nullptr, nullptr);
         std::swap(src, dst);
     }
     *result = src;
@@ -1155,7 +1135,7 @@ void mqr_destroy(mqr_ctx *c) {
     DevBuf<unsigned long long> *u64s[] = {&c->stamp, &c->keysA, &c->keysB, &c->out_off, &c->off_stage,
                                           &c->sortA, &c->sortB};
     for (auto *b : u64s) b->release();
-    DevBuf<uint32_t> *u32s[] = {&c->skey, &c->sid, &c->sort_counts, &c->sort_offs, &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
+    DevBuf<uint32_t> *u32s[] = {&c->skey, &c->sid, &c->sort_counts, &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
                                 &c->leaf_sub_off, &c->leaf_word_off, &c->leaf_item_off,
                                 &c->sub_q, &c->sub_leaf, &c->sub_len, &c->sub_res,
                                 &c->isub, &c->bitmap, &c->item_leaf, &c->up_ids, &c->zmap, &c->pair_q,
@@ -1232,6 +1212,7 @@ mqr_status mqr_create_ex(mqr_rect bounds, const mqr_config *cfg, void *cuda_stre
             return bail(e, "cudaStreamCreate");
         c->own_stream = true;
     }
+    c->small_sort = c->nmax <= kSmallSortMax && small_sort_ready();
     const size_t n = std::max<size_t>(c->nmax, 1);
     if ((e = c->pos.ensure(n)) || (e = c->stamp.ensure(n)) || (e = c->keysA.ensure(n)) ||
         (e = c->keysB.ensure(n)) || (e = c->skey.ensure(n)) || (e = c->sid.ensure(n)) ||
@@ -1239,8 +1220,7 @@ mqr_status mqr_create_ex(mqr_rect bounds, const mqr_config *cfg, void *cuda_stre
         (e = c->leaf_beg.ensure(n + 1)) || (e = c->leaf_nsub.ensure(n)) ||
         (e = c->leaf_sub_off.ensure(n + 1)) || (e = c->leaf_word_off.ensure(n + 1)) ||
         (e = c->leaf_item_off.ensure(n + 1)) ||
-        (e = c->sort_counts.ensure((size_t)256 * ((n + kSortTile - 1) / kSortTile))) ||
-        (e = c->sort_offs.ensure((size_t)256 * ((n + kSortTile - 1) / kSortTile))) ||
+        (e = c->sort_counts.ensure((size_t)256 * sort_tiles((uint32_t)n))) ||
         (e = c->upd_err.ensure(1)) || (e = c->leaf_box.ensure(n)))
         return bail(e, "cudaMalloc (object state)");
     if (cfg->index_kind == MQR_INDEX_QUADTREE && cfg->leaf_cap > (uint32_t)kLeafCapSmem &&

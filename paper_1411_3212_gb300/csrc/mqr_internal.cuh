@@ -118,12 +118,24 @@ struct Worlds {
     uint32_t bits;    // levels above the worlds' roots (4^bits >= n)
 };
 
-// The world of item i: the largest w with base[w] <= i.
-__device__ __forceinline__ uint32_t world_of(uint32_t i, const uint32_t *__restrict__ base, uint32_t n) {
-    uint32_t lo = 0, hi = n;
+// The world of item i: the largest w in [lo, hi) with base[w] <= i (it must lie there).
+__device__ __forceinline__ uint32_t world_of(uint32_t i, const uint32_t *__restrict__ base, uint32_t lo, uint32_t hi) {
     while (hi - lo > 1u) {
         const uint32_t m = (lo + hi) >> 1;
         if (__ldg(base + m) <= i) lo = m; else hi = m;
+    }
+    return lo;
+}
+
+// The same for the whole warp, a 32-way search: every lane gets the world of i.
+__device__ __forceinline__ uint32_t world_of_warp(uint32_t i, const uint32_t *__restrict__ base, uint32_t n) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t lo = 0, hi = n;
+    while (hi - lo > 1u) {
+        const uint32_t step = (hi - lo + 31u) >> 5, m = lo + (lane + 1u) * step;
+        const uint32_t le = __ballot_sync(0xffffffffu, m < hi && __ldg(base + m) <= i);
+        lo += (uint32_t)__popc(le) * step;             // base ascends: the lanes that hold are the first ones
+        hi = min(hi, lo + step);
     }
     return lo;
 }
@@ -274,43 +286,6 @@ __device__ T lookback_warp(T *status, uint32_t tile, T agg, unsigned long long *
     return sum;
 }
 
-// Per-thread look-back for the radix sort, where every thread scans the
-// status of its own digit (consecutive tiles adjacent in memory).
-template <typename T>
-__device__ T lookback1(T *status, uint32_t tile, T agg, unsigned long long *err) {
-    using B = StatusBits<T>;
-    if (tile == 0) {
-        status_store(status, (T(2) << B::kShift) | agg);
-        return T(0);
-    }
-    status_store(status + tile, (T(1) << B::kShift) | agg);
-    T sum = 0;
-    long j = (long)tile - 1;
-    unsigned long long t0 = 0;
-    unsigned spins = 0;
-    while (j >= 0) {
-        const T v = status_load(status + j);
-        const T flag = v >> B::kShift;
-        if (flag == 0) {
-            if ((++spins & 63u) == 0) {
-                const unsigned long long now = global_ns();
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > kWaitNs) {
-                    atomicOr(err, kErrTimeout);
-                    break;
-                }
-            }
-            __nanosleep(32);
-            continue;
-        }
-        sum += v & B::kMask;
-        if (flag == 2) break;
-        --j;
-    }
-    status_store(status + tile, (T(2) << B::kShift) | (sum + agg));
-    return sum;
-}
-
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
@@ -328,34 +303,43 @@ void launch_apply_updates(cudaStream_t st, const uint32_t *ids, const float2 *xy
                           uint32_t nmax, unsigned long long epoch, unsigned long long *stamp,
                           float2 *pos, unsigned long long *err);
 
-// a2: Morton keys of every slot + digit histograms of the 4 sort passes.
+// Start of a tick: the arena (Info first, a multiple of 16 bytes) cleared, the
+// update kernels' error bits or (snap) a snapshot's counters taken over.
+void launch_tick_begin(cudaStream_t st, void *arena, size_t bytes, unsigned long long *upd_err,
+                       const unsigned long long *snap);
+// a2: Morton keys of every slot + the first sort pass's digit counts.
 void launch_state_flags(cudaStream_t st, const unsigned long long *stamp, uint32_t nmax, uint8_t *present);
 void launch_state_stamps(cudaStream_t st, const uint8_t *present, uint32_t nmax, unsigned long long epoch,
                          unsigned long long *stamp);
-// tile_counts: the first sort pass's per-tile digit counts (256 x tiles).
 void launch_morton_keys(cudaStream_t st, const float2 *pos, const unsigned long long *stamp,
                         uint32_t nmax, float x0, float y0, float sx, float sy, Worlds worlds,
-                        unsigned long long *keys, uint32_t *hist4x256, uint32_t *tile_counts, Info *info);
+                        unsigned long long *keys, uint32_t *tile_counts, uint32_t *group_counts, Info *info);
 
-// a3: one onesweep pass over n u64 keys, 8-bit digit at `shift`.  The final
-// pass of the object sort (`final_obj`) writes skey/sid/sxy instead of `out`.
+// a3: one stable radix pass over n u64 keys, 8-bit digit at `shift`, from the
+// per-tile digit counts: tile_counts holds 256 x sort_tiles(n) u32,
+// group_counts sort_group_words(n) u32, zeroed before the pass.  counts_ready:
+// both already hold this pass's counts (the key kernel of the object sort).
+// The final pass of an object sort (final_obj) writes skey/sid and, if sxy is
+// not null, the positions pos[id] to sxy, instead of `out`.
 constexpr int kSortThreads = 512, kSortItems = 8, kSortTile = kSortThreads * kSortItems;
-void launch_onesweep_pass(cudaStream_t st, const unsigned long long *in, unsigned long long *out,
-                          uint32_t n, int shift, const uint32_t *hist256, uint32_t *status,
-                          uint32_t *tile_counter, unsigned long long *err, bool final_obj,
-                          const float2 *pos, uint32_t *skey, uint32_t *sid, float2 *sxy);
-// The same pass without look-back: per-tile digit counts (counts/offs hold
-// 256 x ceil(n / kSortTile) u32 each), a per-digit scan over the tiles, then
-// the rank-and-scatter tile kernel with the precomputed offsets.
-// counts_ready: `counts` already holds the pass's per-tile digit counts.
-void launch_sort_pass_pre(cudaStream_t st, const unsigned long long *in, unsigned long long *out, uint32_t n,
-                          int shift, const uint32_t *hist256, uint32_t *counts, uint32_t *offs,
-                          unsigned long long *err, bool final_obj, const float2 *pos, uint32_t *skey,
-                          uint32_t *sid, float2 *sxy, bool counts_ready);
-// Histograms (nd digit passes at shifts[]) of n u64 keys, for generic sorts.
-void launch_key_histograms(cudaStream_t st, const unsigned long long *keys, uint32_t n,
-                           const int *shifts_host, int nd, uint32_t *hist);
-
+constexpr uint32_t kSortGroup = 32;           // tiles per row of the coarse digit counts
+constexpr uint32_t kSortTotalRows = 8;
+__host__ __device__ constexpr uint32_t sort_tiles(uint32_t n) { return n / kSortTile + (n % kSortTile ? 1u : 0u); }
+__host__ __device__ constexpr uint32_t sort_groups(uint32_t n) { return (sort_tiles(n) + kSortGroup - 1) / kSortGroup; }
+__host__ __device__ constexpr size_t sort_group_words(uint32_t n) { return (size_t)256 * (kSortTotalRows + sort_groups(n)); }
+void launch_sort_pass(cudaStream_t st, const unsigned long long *in, unsigned long long *out, uint32_t n,
+                      int shift, uint32_t *tile_counts, uint32_t *group_counts, bool counts_ready,
+                      unsigned long long *err, bool final_obj, const float2 *pos, uint32_t *skey, uint32_t *sid,
+                      float2 *sxy);
+uint32_t sort_pass_launches(uint32_t n, bool counts_ready);
+// a2 + a3 in one launch (one cluster of blocks) for n <= kSmallSortMax objects;
+// stamp, sxy and info may be null.  small_sort_ready: the current device can
+// run it (called once per device before the first launch).
+constexpr uint32_t kSmallSortMax = 65536;
+bool small_sort_ready();
+cudaError_t launch_small_sort(cudaStream_t st, const float2 *pos, const unsigned long long *stamp, uint32_t n,
+                              float x0, float y0, float sx, float sy, Worlds worlds, uint32_t *skey, uint32_t *sid,
+                              float2 *sxy, Info *info);
 // a4: leaves.  level_mode: 0 = quadtree (capacity rule), 1 = uniform grid at
 // `grid_level`; no leaf above depth min_level (the batched worlds' roots);
 // region_bits > 0: per-region capacities region_cap[4^region_bits] (no leaf
