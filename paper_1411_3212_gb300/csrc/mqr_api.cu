@@ -121,6 +121,11 @@ struct mqr_ctx {
     DevBuf<float4> q_rects;
     DevBuf<unsigned char> out_stage, out_stage2;     // host-output staging (two for the async path)
     DevBuf<unsigned long long> off_stage, off_stage2, sortA, sortB;
+    // sorted kinds: the emitted id lists, per-query offsets of a caller without any, the
+    // queries of long lists, whether the last sorted tick had some
+    DevBuf<uint32_t> list_ids, long_lists;
+    bool had_long_lists = false;
+    DevBuf<unsigned long long> list_off;
     cudaStream_t copy_stream = nullptr;              // device-to-host copies of mqr_tick_host_async
     DevBuf<uint32_t> sid_stage, sid_stage2;          // sorted-id snapshots copied by mqr_get_sorted_async
     cudaEvent_t snap_done = nullptr;
@@ -514,7 +519,7 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     if (admit) {
         // per-query offsets, then the longest prefix of queries that fits
         phase_begin(c, MQR_PHASE_OFFSETS);
-        launch_query_offsets(st, Q, c->qpair.p, c->pair_rec.p, c->out_off.p, offsets, caps, info);
+        launch_query_offsets(st, Q, c->qpair.p, c->pair_rec.p, c->out_off.p, offsets, caps, false, info);
         launch_admit(st, Q, offsets, out ? out_cap_elems : 0, c->qpair.p, c->pair_rec.p, caps, info);
         phase_end(c, MQR_PHASE_OFFSETS, 2);
     }
@@ -528,7 +533,8 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     }
     if (offsets != nullptr && !admit) {
         phase_begin(c, MQR_PHASE_OFFSETS);
-        launch_query_offsets(st, Q, c->qpair.p, c->pair_rec.p, c->out_off.p, offsets, caps, info);
+        launch_query_offsets(st, Q, c->qpair.p, c->pair_rec.p, c->out_off.p, offsets, caps,
+                             emit_kind == kEmitIds && out == c->list_ids.p, info);
         phase_end(c, MQR_PHASE_OFFSETS, 1);
     }
     return check_launch("tick kernels");
@@ -662,15 +668,36 @@ mqr_status enqueue_or_replay(mqr_ctx *c, const float4 *rects, uint32_t Q, int em
     return MQR_OK;
 }
 
+// The sorted kinds' last step: the emitted id lists sorted into the caller's
+// buffer (caps.out = the elements it and the list buffer both hold).
+struct SortedOut {
+    void *out;
+    bool as_pairs;
+};
+
+mqr_status enqueue_list_sort(mqr_ctx *c, uint32_t Q, const unsigned long long *offsets, const SortedOut &so,
+                             const Caps &caps, const Info *info, bool short_lists, bool long_lists) {
+    phase_begin(c, MQR_PHASE_OUTPUT_SORT);
+    if (short_lists)
+        MQR_CUDA(launch_list_sort(c->stream, c->list_ids.p, offsets, Q, so.as_pairs, so.out, c->long_lists.p, caps, info));
+    if (long_lists)
+        MQR_CUDA(launch_long_lists(c->stream, c->num_sms, c->list_ids.p, offsets, so.as_pairs, so.out, c->long_lists.p,
+                                   caps, info));
+    phase_end(c, MQR_PHASE_OUTPUT_SORT, (short_lists && Q ? 1 : 0) + (long_lists ? 1 : 0));
+    return MQR_OK;
+}
+
 // One attempt of a tick (or of a slot's join): enqueue its kernels and the
 // copy of its counters to the host.  Returns after enqueueing.
 mqr_status attempt_enqueue(mqr_ctx *c, const float4 *rects, uint32_t Q, int emit_kind, void *out,
-                           unsigned long long out_cap_elems, unsigned long long *offsets, bool admit, Caps &caps) {
+                           unsigned long long out_cap_elems, unsigned long long *offsets, bool admit, Caps &caps,
+                           const SortedOut *so = nullptr) {
     Arena a = arena_layout(c->nmax, Q, c->sub_q.n, c->cand_tiles);
     MQR_CUDA(c->arena.ensure(a.total));
     caps = Caps{};
     mqr_status s = c->parent ? enqueue_slot(c, rects, Q, emit_kind, out, out_cap_elems, offsets, a, caps)
                              : enqueue_or_replay(c, rects, Q, emit_kind, out, out_cap_elems, offsets, a, caps, admit);
+    if (s == MQR_OK && so) s = enqueue_list_sort(c, Q, offsets, *so, caps, at<Info>(c, a.info), true, c->had_long_lists);
     if (s != MQR_OK) return s;
     MQR_CUDA(cudaMemcpyAsync(c->info_host, c->arena.p + a.info, sizeof(Info), cudaMemcpyDeviceToHost, c->stream));
     return MQR_OK;
@@ -729,13 +756,14 @@ mqr_status attempt_check(mqr_ctx *c, uint32_t Q, int emit_kind, const Caps &caps
 // tick's device state valid and c->last filled.  `out` may be null (then
 // nothing is emitted).  admit: see enqueue_join.
 mqr_status run_tick(mqr_ctx *c, const float4 *rects, uint32_t Q, int emit_kind, void *out,
-                    unsigned long long out_cap_elems, unsigned long long *offsets, bool admit = false) {
+                    unsigned long long out_cap_elems, unsigned long long *offsets, bool admit = false,
+                    const SortedOut *so = nullptr) {
     mqr_status s = ensure_tick_buffers(c, Q);
     if (s != MQR_OK) return s;
     c->retries = 0;
     for (int attempt = 0; attempt < 8; ++attempt) {
         Caps caps{};
-        s = attempt_enqueue(c, rects, Q, emit_kind, out, out_cap_elems, offsets, admit, caps);
+        s = attempt_enqueue(c, rects, Q, emit_kind, out, out_cap_elems, offsets, admit, caps, so);
         if (s != MQR_OK) return s;
         MQR_CUDA(cudaStreamSynchronize(c->stream));
         bool again = false;
@@ -862,34 +890,72 @@ mqr_status tick_device_impl(mqr_ctx *c, const float *rects_dev, uint32_t Q, int 
             return fail(MQR_ERR_CAPACITY, "output buffer too small for the tick's results");
         return MQR_OK;
     }
-    // sorted kinds: count first, then emit (qidx, id) keys, sort, lay out.
-    mqr_status s = run_tick(c, rects, Q, -1, nullptr, 0, offs);
+    // sorted kinds: the id lists are emitted to a buffer of the context and
+    // every list sorted into the caller's.  The first tick only counts (with
+    // no list buffer yet, or one that is too small, nothing is emitted); a
+    // later one whose lists fit the buffer left by it is answered in one go,
+    // its long lists too if the tick before had some (else they follow).
+    const bool as_pairs = kind == MQR_OUT_PAIRS_SORTED;
+    const size_t eb = out_elem_bytes(kind);
+    if (!offs) {
+        MQR_CUDA(c->list_off.ensure((size_t)Q + 1));
+        offs = c->list_off.p;
+    }
+    MQR_CUDA(c->list_ids.ensure(4096));
+    MQR_CUDA(c->long_lists.ensure((size_t)Q + 2));
+    const SortedOut so{out_dev, as_pairs};
+    const unsigned long long fits = out_dev ? std::min<unsigned long long>(c->list_ids.n, cap_bytes / eb) : 0;
+    mqr_status s = run_tick(c, rects, Q, kEmitIds, c->list_ids.p, fits, offs, false, &so);
     *out_count = c->last.n_results;
     if (s != MQR_OK) return s;
     const uint64_t R = c->last.n_results;
-    const size_t eb = out_elem_bytes(kind);
     if (R > cap_bytes / eb || (R && out_dev == nullptr))
         return fail(MQR_ERR_CAPACITY, "output buffer too small for the tick's results");
     if (R >= (1ull << 30)) return fail(MQR_ERR_INVALID_ARG, "sorted output kinds are limited to R < 2^30");
-    if (R == 0) return MQR_OK;
-    MQR_CUDA(c->sortA.ensure(R));
-    MQR_CUDA(c->sortB.ensure(R));
+    const bool by_lists = c->last.max_list <= (unsigned long long)kBlockList;
+    const bool done_long = c->had_long_lists;
+    const bool any_long = c->had_long_lists = by_lists && c->last.max_list > (unsigned long long)kMidList;
+    if (R == 0 || (by_lists && R <= fits && (done_long || !any_long))) return MQR_OK;
+    // emit again: into a list buffer that holds everything, or as (qidx, id)
+    // keys for the radix sort when a list is longer than the list sort takes
+    if (by_lists) {
+        if (R > fits) MQR_CUDA(c->list_ids.ensure(grow_to(R)));
+    } else {
+        MQR_CUDA(c->sortA.ensure(R));
+        MQR_CUDA(c->sortB.ensure(R));
+    }
     Arena a = arena_layout(c->nmax, Q, c->sub_q.n, c->cand_tiles);
     Caps caps{c->sub_q.n, c->isub.n, std::min<size_t>(c->bitmap.n, 0xffffffffull), R, c->cand_tiles,
               c->item_leaf.n};
     Info *info = at<Info>(c, a.info);
-    phase_begin(c, MQR_PHASE_OUTPUT_SORT);
-    launch_emit(c->stream, c->num_sms * (int)c->bps_emit, kEmitKeys64, c->sub_q.p, c->sub_leaf.p, c->sub_len.p,
-                c->leaf_word_off.p, c->out_off.p, c->leaf_beg.p, c->sid.p, c->bitmap.p, c->sortA.p, wpr,
-                at<uint32_t>(c, a.counters) + 9, caps, info);
-    s = check_launch("emit keys");
+    if (by_lists && R <= fits) {                     // only the long lists are left
+        caps.out = fits;
+        s = enqueue_list_sort(c, Q, offs, so, caps, info, false, true);
+        if (s != MQR_OK) return s;
+        MQR_CUDA(cudaStreamSynchronize(c->stream));
+        phases_collect(c, false);
+        return MQR_OK;
+    }
+    uint32_t *ticket = at<uint32_t>(c, a.counters) + 9;
+    MQR_CUDA(cudaMemsetAsync(ticket, 0, sizeof(uint32_t), c->stream));
+    phase_begin(c, MQR_PHASE_EMIT);
+    launch_emit(c->stream, c->num_sms * (int)c->bps_emit, by_lists ? kEmitIds : kEmitKeys64, c->sub_q.p, c->sub_leaf.p,
+                c->sub_len.p, c->leaf_word_off.p, c->out_off.p, c->leaf_beg.p, c->sid.p, c->bitmap.p,
+                by_lists ? (void *)c->list_ids.p : (void *)c->sortA.p, wpr, ticket, caps, info);
+    phase_end(c, MQR_PHASE_EMIT, 1);
+    s = check_launch("emit lists");
     if (s != MQR_OK) return s;
-    unsigned long long *sorted = nullptr;
-    s = sort_result_keys(c, R, Q, &sorted);
-    if (s != MQR_OK) return s;
-    launch_keys_to_output(c->stream, sorted, R, kind == MQR_OUT_PAIRS_SORTED, out_dev);
-    phase_end(c, MQR_PHASE_OUTPUT_SORT, 0);
-    s = check_launch("layout");
+    if (by_lists) {
+        s = enqueue_list_sort(c, Q, offs, so, caps, info, true, any_long);
+    } else {
+        unsigned long long *sorted = nullptr;
+        phase_begin(c, MQR_PHASE_OUTPUT_SORT);
+        s = sort_result_keys(c, R, Q, &sorted);
+        if (s != MQR_OK) return s;
+        launch_keys_to_output(c->stream, sorted, R, as_pairs, out_dev);
+        phase_end(c, MQR_PHASE_OUTPUT_SORT, 0);
+        s = check_launch("layout");
+    }
     if (s != MQR_OK) return s;
     MQR_CUDA(cudaStreamSynchronize(c->stream));
     phases_collect(c, false);
@@ -921,7 +987,8 @@ const char *mqr_last_error(void) { return g_err.c_str(); }
 struct mqr_cost {
     int device = 0;
     cudaStream_t stream = nullptr;
-    DevBuf<float> params, m, v, X, y, out, loss;
+    int num_sms = 0;
+    DevBuf<float> params, m, v, X, y, out, loss, scratch;
     uint32_t steps = 0;
 };
 
@@ -1133,9 +1200,9 @@ void mqr_destroy(mqr_ctx *c) {
     c->region_stats.release();
     c->state_flags.release();
     DevBuf<unsigned long long> *u64s[] = {&c->stamp, &c->keysA, &c->keysB, &c->out_off, &c->off_stage,
-                                          &c->sortA, &c->sortB};
+                                          &c->sortA, &c->sortB, &c->list_off};
     for (auto *b : u64s) b->release();
-    DevBuf<uint32_t> *u32s[] = {&c->skey, &c->sid, &c->sort_counts, &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
+    DevBuf<uint32_t> *u32s[] = {&c->list_ids, &c->long_lists, &c->skey, &c->sid, &c->sort_counts, &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
                                 &c->leaf_sub_off, &c->leaf_word_off, &c->leaf_item_off,
                                 &c->sub_q, &c->sub_leaf, &c->sub_len, &c->sub_res,
                                 &c->isub, &c->bitmap, &c->item_leaf, &c->up_ids, &c->zmap, &c->pair_q,

@@ -55,6 +55,7 @@ struct Info {
     unsigned long long emit_end;     // admission: 0 = emit all, else (bit 63 |) emit records [0, low 32 bits) only
     unsigned long long admitted;     // admission: queries [0, admitted) answered
     unsigned long long admitted_out; // admission: their output elements
+    unsigned long long max_list;     // sorted kinds: the longest query's results
 };
 
 // Capacities of the growable per-tick buffers (host-chosen, passed by value).
@@ -456,8 +457,18 @@ void launch_admit(cudaStream_t st, uint32_t Q, const unsigned long long *offsets
 
 // Per-query offsets: off[q] = out_off[pair_rec[qpair[q]]].
 void launch_query_offsets(cudaStream_t st, uint32_t Q, const uint32_t *qpair, const uint32_t *pair_rec,
-                          const unsigned long long *out_off, unsigned long long *offsets, Caps caps,
-                          const Info *info);
+                          const unsigned long long *out_off, unsigned long long *offsets, Caps caps, bool longest,
+                          Info *info);
+
+// Sorted kinds: every query's ids (ids[offsets[q] .. offsets[q + 1])) sorted into
+// `out`, if no list is longer than kBlockList (info->max_list) and the tick's
+// output fits caps.out; lists above kMidList by the second launch, which may
+// follow any time later.  long_lists holds Q + 2 words.
+constexpr int kMidList = 4096, kBlockList = 16384;
+cudaError_t launch_list_sort(cudaStream_t st, const uint32_t *ids, const unsigned long long *offsets, uint32_t Q,
+                             bool as_pairs, void *out, uint32_t *long_lists, Caps caps, const Info *info);
+cudaError_t launch_long_lists(cudaStream_t st, int num_sms, const uint32_t *ids, const unsigned long long *offsets,
+                              bool as_pairs, void *out, uint32_t *long_lists, Caps caps, const Info *info);
 
 // (qidx << 32 | id) keys -> pairs (qidx, id) or ids.
 void launch_keys_to_output(cudaStream_t st, const unsigned long long *keys, uint64_t n,
