@@ -413,7 +413,7 @@ mqr_status mqr_region_work(mqr_ctx *ctx, const float *rects_dev, uint32_t Q, uin
 
 /* Learned tick-cost model: a multilayer perceptron 5 -> 64 -> 64 -> 1 with
  * ReLU hidden layers, trained on the device (hand-written forward, backward
- * and Adam kernels, one block) to map tick features to the logarithm of the
+ * and Adam kernels) to map tick features to the logarithm of the
  * tick's time, so that a caller can pick the index configuration of the next
  * tick (mqr_set_index).  The paper models its phases' costs analytically
  * (the filtering complexity of Sec. 5.4); this learns the cost from

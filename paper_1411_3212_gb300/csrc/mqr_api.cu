@@ -992,6 +992,30 @@ struct mqr_cost {
     uint32_t steps = 0;
 };
 
+// One training (or, with grad, gradient) launch and its results: the loss and
+// whether the kernel's barrier ran out of time.
+static mqr_status cost_run(mqr_cost *m, const float *X_host, const float *y_host, uint32_t n, uint32_t epochs, float lr,
+                           float *grad_dev, float *grad_host, float *loss_out) {
+    MQR_CUDA(m->X.ensure((size_t)n * 5));
+    MQR_CUDA(m->y.ensure(n));
+    MQR_CUDA(m->scratch.ensure(cost_train_scratch_floats(n, m->num_sms)));
+    MQR_CUDA(cudaMemcpyAsync(m->X.p, X_host, (size_t)n * 5 * 4, cudaMemcpyHostToDevice, m->stream));
+    MQR_CUDA(cudaMemcpyAsync(m->y.p, y_host, (size_t)n * 4, cudaMemcpyHostToDevice, m->stream));
+    uint32_t *sync = nullptr, gave_up[2] = {0, 0};
+    MQR_CUDA(launch_cost_train(m->stream, m->num_sms, m->params.p, m->m.p, m->v.p, m->steps, m->X.p, m->y.p, n, epochs,
+                               lr, m->loss.p, grad_dev, m->scratch.p, &sync));
+    if (!grad_dev) m->steps += epochs;
+    float l = 0.f;
+    if (grad_dev)
+        MQR_CUDA(cudaMemcpyAsync(grad_host, grad_dev, cost_param_count() * 4, cudaMemcpyDeviceToHost, m->stream));
+    MQR_CUDA(cudaMemcpyAsync(&l, m->loss.p, 4, cudaMemcpyDeviceToHost, m->stream));
+    MQR_CUDA(cudaMemcpyAsync(gave_up, sync, sizeof(gave_up), cudaMemcpyDeviceToHost, m->stream));
+    MQR_CUDA(cudaStreamSynchronize(m->stream));
+    if (gave_up[1]) return fail(MQR_ERR_TIMEOUT, "a device-side wait exceeded its deadline");
+    if (loss_out) *loss_out = l;
+    return MQR_OK;
+}
+
 uint32_t mqr_cost_param_count(void) { return (uint32_t)cost_param_count(); }
 
 mqr_status mqr_cost_create(mqr_cost **out) {
@@ -1005,6 +1029,7 @@ mqr_status mqr_cost_create(mqr_cost **out) {
     if (e == cudaSuccess) e = m->params.ensure(P);
     if (e == cudaSuccess) e = m->m.ensure(P);
     if (e == cudaSuccess) e = m->v.ensure(P);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, m->device);
     if (e == cudaSuccess) e = m->loss.ensure(1);
     if (e == cudaSuccess) e = cudaMemset(m->params.p, 0, P * 4);
     if (e == cudaSuccess) e = cudaMemset(m->m.p, 0, P * 4);
@@ -1043,39 +1068,16 @@ mqr_status mqr_cost_train(mqr_cost *m, const float *X_host, const float *y_host,
     if (n == 0 || epochs == 0) return MQR_OK;
     if (!(lr > 0.f)) return fail(MQR_ERR_INVALID_ARG, "lr must be > 0");
     MQR_CUDA(cudaSetDevice(m->device));
-    MQR_CUDA(m->X.ensure((size_t)n * 5));
-    MQR_CUDA(m->y.ensure(n));
-    MQR_CUDA(cudaMemcpyAsync(m->X.p, X_host, (size_t)n * 5 * 4, cudaMemcpyHostToDevice, m->stream));
-    MQR_CUDA(cudaMemcpyAsync(m->y.p, y_host, (size_t)n * 4, cudaMemcpyHostToDevice, m->stream));
-    MQR_CUDA(launch_cost_train(m->stream, m->params.p, m->m.p, m->v.p, m->steps, m->X.p, m->y.p, n, epochs, lr,
-                               m->loss.p, nullptr));
-    m->steps += epochs;
-    float l = 0.f;
-    MQR_CUDA(cudaMemcpyAsync(&l, m->loss.p, 4, cudaMemcpyDeviceToHost, m->stream));
-    MQR_CUDA(cudaStreamSynchronize(m->stream));
-    if (loss_out) *loss_out = l;
-    return MQR_OK;
+    return cost_run(m, X_host, y_host, n, epochs, lr, nullptr, nullptr, loss_out);
 }
 
 mqr_status mqr_cost_gradient(mqr_cost *m, const float *X_host, const float *y_host, uint32_t n, float *grad_host,
                              float *loss_out) {
     if (!m || !grad_host || (n && (!X_host || !y_host))) return fail(MQR_ERR_INVALID_ARG, "NULL argument");
     if (n == 0) return fail(MQR_ERR_INVALID_ARG, "n must be >= 1");
-    const size_t P = cost_param_count();
     MQR_CUDA(cudaSetDevice(m->device));
-    MQR_CUDA(m->X.ensure((size_t)n * 5));
-    MQR_CUDA(m->y.ensure(n));
-    MQR_CUDA(m->out.ensure(std::max<size_t>(P, n)));
-    MQR_CUDA(cudaMemcpyAsync(m->X.p, X_host, (size_t)n * 5 * 4, cudaMemcpyHostToDevice, m->stream));
-    MQR_CUDA(cudaMemcpyAsync(m->y.p, y_host, (size_t)n * 4, cudaMemcpyHostToDevice, m->stream));
-    MQR_CUDA(launch_cost_train(m->stream, m->params.p, m->m.p, m->v.p, m->steps, m->X.p, m->y.p, n, 1, 1.f,
-                               m->loss.p, m->out.p));
-    float l = 0.f;
-    MQR_CUDA(cudaMemcpyAsync(grad_host, m->out.p, P * 4, cudaMemcpyDeviceToHost, m->stream));
-    MQR_CUDA(cudaMemcpyAsync(&l, m->loss.p, 4, cudaMemcpyDeviceToHost, m->stream));
-    MQR_CUDA(cudaStreamSynchronize(m->stream));
-    if (loss_out) *loss_out = l;
-    return MQR_OK;
+    MQR_CUDA(m->out.ensure(std::max<size_t>(cost_param_count(), n)));
+    return cost_run(m, X_host, y_host, n, 1, 1.f, m->out.p, grad_host, loss_out);
 }
 
 mqr_status mqr_cost_predict(mqr_cost *m, const float *X_host, uint32_t n, float *out_host) {
@@ -1096,7 +1098,7 @@ void mqr_cost_destroy(mqr_cost *m) {
     cudaSetDevice(m->device);
     if (m->stream) cudaStreamSynchronize(m->stream);
     m->params.release(); m->m.release(); m->v.release(); m->X.release(); m->y.release();
-    m->out.release(); m->loss.release();
+    m->out.release(); m->loss.release(); m->scratch.release();
     if (m->stream) cudaStreamDestroy(m->stream);
     delete m;
 }

@@ -447,8 +447,10 @@ void launch_atomic_baseline(cudaStream_t st, int num_sms, const float4 *rects, c
 
 // Learned tick-cost model (k_cost.cu): MLP 5 -> 64 -> 64 -> 1.
 size_t cost_param_count();
-cudaError_t launch_cost_train(cudaStream_t st, float *params, float *m, float *v, uint32_t step0, const float *X,
-                              const float *y, uint32_t n, uint32_t epochs, float lr, float *loss, float *grad);
+size_t cost_train_scratch_floats(uint32_t n, int num_sms);
+cudaError_t launch_cost_train(cudaStream_t st, int num_sms, float *params, float *m, float *v, uint32_t step0,
+                              const float *X, const float *y, uint32_t n, uint32_t epochs, float lr, float *loss,
+                              float *grad, float *scratch, uint32_t **sync_out);
 cudaError_t launch_cost_predict(cudaStream_t st, const float *params, const float *X, uint32_t n, float *out);
 
 // Admission by output memory: queries [0, A) whose output fits cap elements.
