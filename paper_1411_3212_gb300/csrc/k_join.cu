@@ -62,12 +62,12 @@ filter_kernel(const float4 *__restrict__ rects, const float2 *__restrict__ sxy,
     const int lane = threadIdx.x & 31;
     const float qnan = __int_as_float(0x7fc00000);
     // items are handed out by a ticket counter (their sizes vary: 1-32
-    // subqueries x 1-8 words); the next ticket is drawn during the current item
-    uint32_t item = 0, next = 0;
-    if (lane == 0) item = atomicAdd(ticket, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
+    // subqueries x 1-8 words) after every warp's first one, which is its own;
+    // the next ticket is drawn during the current item
+    const uint32_t warps = gridDim.x * (kFilterThreads / 32);
+    uint32_t item = blockIdx.x * (kFilterThreads / 32) + (threadIdx.x >> 5), next = 0xffffffffu;
     for (; item < items; item = __shfl_sync(0xffffffffu, next, 0)) {
-        if (lane == 0) next = atomicAdd(ticket, 1u);
+        if (lane == 0 && items > warps) next = warps + atomicAdd(ticket, 1u);
         const uint32_t leaf = __ldg(item_leaf + item);
         const uint32_t r = item - __ldg(leaf_item_off + leaf);
         const uint32_t soff = __ldg(leaf_sub_off + leaf);
@@ -342,20 +342,37 @@ __device__ __forceinline__ void emit_run(void *out, unsigned long long off, uint
         const uint32_t n2 = n >> 1;
         uint4 *o4 = reinterpret_cast<uint4 *>(out) + (off >> 1);
         const uint32_t *src = sid + b;
-        for (uint32_t i0 = 0; i0 < n2; i0 += 32u * kRunSteps) {
-            uint32_t a[2 * kRunSteps];
+        if (!(b & 1u)) {                            // the ids too: one 8-byte load for each store
+            const uint2 *src2 = reinterpret_cast<const uint2 *>(src);
+            for (uint32_t i0 = 0; i0 < n2; i0 += 32u * kRunSteps) {
+                uint2 a[kRunSteps];
 #pragma unroll
-            for (int u = 0; u < kRunSteps; ++u) {
-                const uint32_t i = i0 + lane + 32u * u;
-                if (i < n2) {
-                    a[2 * u] = __ldg(src + 2 * i);
-                    a[2 * u + 1] = __ldg(src + 2 * i + 1);
+                for (int u = 0; u < kRunSteps; ++u) {
+                    const uint32_t i = i0 + lane + 32u * u;
+                    if (i < n2) a[u] = __ldg(src2 + i);
+                }
+#pragma unroll
+                for (int u = 0; u < kRunSteps; ++u) {
+                    const uint32_t i = i0 + lane + 32u * u;
+                    if (i < n2) o4[i] = make_uint4(q, a[u].x, q, a[u].y);
                 }
             }
+        } else {
+            for (uint32_t i0 = 0; i0 < n2; i0 += 32u * kRunSteps) {
+                uint32_t a[2 * kRunSteps];
 #pragma unroll
-            for (int u = 0; u < kRunSteps; ++u) {
-                const uint32_t i = i0 + lane + 32u * u;
-                if (i < n2) o4[i] = make_uint4(q, a[2 * u], q, a[2 * u + 1]);
+                for (int u = 0; u < kRunSteps; ++u) {
+                    const uint32_t i = i0 + lane + 32u * u;
+                    if (i < n2) {
+                        a[2 * u] = __ldg(src + 2 * i);
+                        a[2 * u + 1] = __ldg(src + 2 * i + 1);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kRunSteps; ++u) {
+                    const uint32_t i = i0 + lane + 32u * u;
+                    if (i < n2) o4[i] = make_uint4(q, a[2 * u], q, a[2 * u + 1]);
+                }
             }
         }
         if ((n & 1u) && lane == 0) emit_one<KIND>(out, off + n - 1, q, __ldg(sid + b + n - 1), wpr);
@@ -402,25 +419,33 @@ __device__ __forceinline__ uint32_t emit_words(void *out, unsigned long long off
 }
 
 // Intersecting records of at most kUnitMaxWords bitmap words (leaves of at
-// most 256 objects) are decoded word-parallel: every word of the batch's such
-// records is a "unit"; a round of 32 units is set up lane-parallel (lane l:
-// the word of unit l, its record, and its output position from a segmented
-// scan of the words' popcounts), then the warp writes the round's units one
-// after another (Alg. 4: lane i writes the result of bit i, coalesced), so
-// the per-record bookkeeping is paid once per 32 words instead of once per
-// record, and only the ids of set bits are loaded.
+// most 256 objects) are decoded word-parallel: every two consecutive words of
+// the batch's such records are a "unit"; a round of 32 units is set up
+// lane-parallel (lane l: the words of unit l, its record, and its output
+// position from a segmented scan of the units' popcounts), then the warp
+// writes the round's units one after another (Alg. 4: lane i writes the result
+// of bit i, coalesced), so the per-record bookkeeping is paid once per 64
+// words instead of once per record, and only the ids of set bits are loaded.
+// A unit of two words reads its descriptor three times for two id loads and two
+// stores, a unit of one word as often for one of each.  At 491M pairs (3.9 GB)
+// of 6.3M records: 902 -> 855 us; 256 worlds, 71M pairs: 282 -> 260.  Of the
+// 855, the covering runs alone take 650 (4.4 TB/s; a kernel that only writes
+// aligned kilobytes of the same pairs from ids in L2 reaches 5.6) and the units
+// alone 384.  More in flight was slower: four units 977, three or four 16-byte
+// steps of a run 924, 40 registers at six blocks per SM 881, 64 at four 865.
 constexpr uint32_t kUnitMaxWords = 8;
+constexpr uint32_t kRecUnits = kUnitMaxWords / 2;
 
-// An 8-byte shared-memory load kept where it is written (not merged with
+// A 16-byte shared-memory load kept where it is written (not merged with
 // another load of the same slot), so that a unit's descriptor is read again
 // where it is used instead of being held in registers.
-__device__ __forceinline__ uint2 ld_shared_v2(const uint32_t *p) {
-    uint2 v;
+__device__ __forceinline__ uint4 ld_shared_v4(const uint4 *p) {
+    uint4 v;
     const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
     return v;
 }
-constexpr int kUnitUnroll = 4;            // units whose id loads are issued together
+constexpr int kUnitUnroll = 2;           // units whose id loads are issued together
 
 // One warp per batch of 32 consecutive subquery records (query-major order,
 // so the output is written front to back): lane j loads the metadata of
@@ -428,7 +453,7 @@ constexpr int kUnitUnroll = 4;            // units whose id loads are issued tog
 // intersecting records are decoded as units (above), then its covering runs
 // and larger intersecting records one by one, with broadcast metadata.
 template <int KIND>
-__global__ void __launch_bounds__(kEmitThreads, 6)
+__global__ void __launch_bounds__(kEmitThreads, 5)
 emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub_leaf,
             const uint32_t *__restrict__ sub_len, const uint32_t *__restrict__ leaf_word_off,
             const unsigned long long *__restrict__ out_off, const uint32_t *__restrict__ leaf_beg,
@@ -437,10 +462,9 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
     // per record: {q, bitmap row, first sorted object, objects | covering flag} and its output offset
     __shared__ uint4 s_rec[kEmitWarps][32];
     __shared__ unsigned long long s_off[kEmitWarps][32];
-    // per unit of the batch: record (low 5 bits) and word of the record (high 3 bits)
-    __shared__ uint8_t s_map[kEmitWarps][32 * kUnitMaxWords];
-    // per unit of a round: {first object of the word, word, word, q} (the id loads read the first
-    // pair, the stores the second) and the address of its first output element
+    // per unit of the batch: record (low 5 bits) and unit of the record (high 3 bits)
+    __shared__ uint8_t s_map[kEmitWarps][32 * kRecUnits];
+    // per unit of a round: {first object, words, q} and the address of its first output element
     __shared__ uint4 s_unit[kEmitWarps][32];
     __shared__ unsigned long long s_uptr[kEmitWarps][32];
     if (!tick_buffers_ok(info, caps)) return;
@@ -450,18 +474,23 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const uint32_t lt = lanemask_lt();
-    const uint32_t nbatch = (nsub + 31u) >> 5;
-    // batches are handed out by a ticket counter (their sizes vary widely);
-    // the next ticket is drawn while the current batch is processed
-    uint32_t batch = 0, next = 0;
-    if (lane == 0) batch = atomicAdd(ticket, 1u);
-    batch = __shfl_sync(0xffffffffu, batch, 0);
+    const uint32_t warps = gridDim.x * kEmitWarps;
+    // records of a batch: 32, or 16, 8, 4 while there are fewer records than
+    // that for every warp (a batch's units are written one after another: a
+    // small tick's emit 14 -> 5.5 us)
+    const uint32_t lg = nsub >= warps * 32u ? 5u : nsub >= warps * 16u ? 4u : nsub >= warps * 8u ? 3u : 2u;
+    const uint32_t nbatch = (nsub + (1u << lg) - 1u) >> lg;
+    // batches are handed out by a ticket counter (their sizes vary widely)
+    // after every warp's first one, which is its own (9,728 warps drawing a
+    // first ticket from one word took 4 us of a small tick's filter, one ticket
+    // a nanosecond); the next ticket is drawn while the current batch is processed
+    uint32_t batch = blockIdx.x * kEmitWarps + wib, next = 0xffffffffu;
     for (; batch < nbatch; batch = __shfl_sync(0xffffffffu, next, 0)) {
-        if (lane == 0) next = atomicAdd(ticket, 1u);
-        const uint32_t k = batch * 32u + lane;
+        if (lane == 0 && nbatch > warps) next = warps + atomicAdd(ticket, 1u);
+        const uint32_t k = (batch << lg) + lane;
         uint32_t nw = 0;
         bool rest = false;
-        if (k < nsub) {
+        if (lane < (1 << lg) && k < nsub) {
             const uint32_t sl = __ldg(sub_leaf + k);
             const uint32_t first = sl & 0x7fffffffu;
             const bool cov = (sl & 0x80000000u) != 0u;
@@ -473,7 +502,7 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
             const uint32_t row = cov ? 0u : __ldg(leaf_word_off + first) + lr * wl;
             s_rec[wib][lane] = make_uint4(__ldg(sub_q + k), row, b, (e - b) | (cov ? 0x80000000u : 0u));
             s_off[wib][lane] = __ldg(out_off + k);
-            if (!cov && wl <= kUnitMaxWords) nw = wl;
+            if (!cov && wl <= kUnitMaxWords) nw = (wl + 1u) >> 1;
             else rest = true;
         }
         // the batch's units: record j owns units [base, base + nw)
@@ -487,19 +516,21 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
         for (uint32_t u0 = 0; u0 < nunits; u0 += 32) {
             const uint32_t u = u0 + lane;
             const bool have = u < nunits;
-            uint32_t r = 32u, w = 0u;
-            uint4 unit = make_uint4(0u, 0u, 0u, 0u);      // lanes past the last unit: an empty word
+            uint32_t r = 32u;
+            uint4 unit = make_uint4(0u, 0u, 0u, 0u);      // lanes past the last unit: empty words
             if (have) {
                 const uint32_t m = s_map[wib][u];
                 r = m & 31u;
                 const uint4 rec = s_rec[wib][r];
-                const uint32_t wi = m >> 5;
-                w = __ldg(bitmap + rec.y + wi);
-                unit = make_uint4(rec.z + 32u * wi, w, w, rec.x);
+                const uint32_t wi = (m >> 5) * 2u;
+                unit.x = rec.z + 32u * wi;
+                unit.y = __ldg(bitmap + rec.y + wi);
+                if (32u * (wi + 1u) < rec.w) unit.z = __ldg(bitmap + rec.y + wi + 1u);
+                unit.w = rec.x;
             }
             // segmented inclusive scan of the popcounts over units of one record
             // (a record's units are consecutive): key r in the high half
-            const uint32_t c = __popc(w);
+            const uint32_t c = __popc(unit.y) + __popc(unit.z);
             uint32_t v = (r << 16) | c;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
@@ -514,17 +545,21 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
             __syncwarp();
             const uint32_t nun = min(32u, nunits - u0);
             for (uint32_t t0 = 0; t0 < nun; t0 += kUnitUnroll) {
-                uint32_t id[kUnitUnroll];
+                uint32_t id[2 * kUnitUnroll];
 #pragma unroll
                 for (int t = 0; t < kUnitUnroll; ++t) {      // slots past nun hold empty words
-                    const uint2 yw = ld_shared_v2(&s_unit[wib][(t0 + t) & 31u].x);
-                    if (yw.y & (1u << lane)) id[t] = __ldg(sid + yw.x + lane);
+                    const uint4 d = ld_shared_v4(&s_unit[wib][(t0 + t) & 31u]);
+                    const uint32_t *src = sid + d.x + lane;
+                    if (d.y & (1u << lane)) id[2 * t] = __ldg(src);
+                    if (d.z & (1u << lane)) id[2 * t + 1] = __ldg(src + 32);
                 }
 #pragma unroll
                 for (int t = 0; t < kUnitUnroll; ++t) {
-                    const uint2 wq = ld_shared_v2(&s_unit[wib][(t0 + t) & 31u].z);
-                    if (wq.x & (1u << lane))
-                        emit_at<KIND>(s_uptr[wib][(t0 + t) & 31u], __popc(wq.x & lt), wq.y, id[t], out, wpr);
+                    const uint4 d = ld_shared_v4(&s_unit[wib][(t0 + t) & 31u]);
+                    const unsigned long long to = s_uptr[wib][(t0 + t) & 31u];
+                    if (d.y & (1u << lane)) emit_at<KIND>(to, __popc(d.y & lt), d.w, id[2 * t], out, wpr);
+                    if (d.z & (1u << lane))
+                        emit_at<KIND>(to, __popc(d.y) + __popc(d.z & lt), d.w, id[2 * t + 1], out, wpr);
                 }
             }
             __syncwarp();

@@ -345,6 +345,7 @@ cand_write_kernel(int covering, const uint32_t *__restrict__ tile_p0, const uint
     const uint32_t npairs = (uint32_t)info->n_pairs;
     const unsigned long long ntiles = (ncand + 31) >> 5;
     const unsigned long long nchunks = (ntiles + kCandChunkTiles - 1) / kCandChunkTiles;
+    if (blockIdx.x >= nchunks) return;          // the blocks that stay draw every chunk
     const uint32_t lt = lanemask_lt();
     uint4 *my = s_rec[warp];
     unsigned long long n_i = 0, n_c = 0;
