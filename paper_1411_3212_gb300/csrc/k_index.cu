@@ -16,38 +16,62 @@ namespace mqr {
 // largest stamp of the call wins (later call = larger epoch), then only the
 // winning update writes the position.
 // ---------------------------------------------------------------------------
-__global__ void stamp_kernel(const uint32_t *__restrict__ ids, uint32_t n, uint32_t nmax,
-                             unsigned long long epoch, unsigned long long *__restrict__ stamp,
-                             unsigned long long *err) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint32_t id = ids[i];
-    if (id >= nmax) {
-        atomicOr(err, kErrBadId);
-        return;
+//
+// Four updates of a thread are in flight (a block apart, so that every load is
+// coalesced): both kernels wait on memory, the second on two dependent steps.
+constexpr uint32_t kUpdThreads = 256, kUpdItems = 4;
+
+__global__ void __launch_bounds__(kUpdThreads)
+stamp_kernel(const uint32_t *__restrict__ ids, uint32_t n, uint32_t nmax,
+             unsigned long long epoch, unsigned long long *__restrict__ stamp, unsigned long long *err) {
+    const uint32_t i0 = blockIdx.x * (kUpdThreads * kUpdItems) + threadIdx.x;
+    if (i0 >= n) return;
+    const uint32_t left = n - i0;
+    uint32_t id[kUpdItems];
+#pragma unroll
+    for (uint32_t u = 0; u < kUpdItems; ++u)
+        if (u * kUpdThreads < left) id[u] = __ldg(ids + i0 + u * kUpdThreads);
+#pragma unroll
+    for (uint32_t u = 0; u < kUpdItems; ++u) {
+        if (u * kUpdThreads >= left) break;
+        if (id[u] >= nmax) atomicOr(err, kErrBadId);
+        else atomicMax(stamp + id[u], (epoch << 32) | (i0 + u * kUpdThreads));
     }
-    atomicMax(stamp + id, (epoch << 32) | i);
 }
 
-__global__ void write_winner_kernel(const uint32_t *__restrict__ ids, const float2 *__restrict__ xy,
-                                    uint32_t n, uint32_t nmax, unsigned long long epoch,
-                                    const unsigned long long *__restrict__ stamp,
-                                    float2 *__restrict__ pos) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint32_t id = ids[i];
-    if (id >= nmax) return;
-    if (stamp[id] == ((epoch << 32) | i)) pos[id] = xy[i];
+__global__ void __launch_bounds__(kUpdThreads)
+write_winner_kernel(const uint32_t *__restrict__ ids, const float2 *__restrict__ xy,
+                    uint32_t n, uint32_t nmax, unsigned long long epoch,
+                    const unsigned long long *__restrict__ stamp, float2 *__restrict__ pos) {
+    const uint32_t i0 = blockIdx.x * (kUpdThreads * kUpdItems) + threadIdx.x;
+    if (i0 >= n) return;
+    const uint32_t left = n - i0;
+    uint32_t id[kUpdItems];
+    float2 v[kUpdItems];
+    unsigned long long s[kUpdItems];
+#pragma unroll
+    for (uint32_t u = 0; u < kUpdItems; ++u) {
+        id[u] = 0xffffffffu;
+        if (u * kUpdThreads < left) {
+            id[u] = __ldg(ids + i0 + u * kUpdThreads);
+            v[u] = __ldg(xy + i0 + u * kUpdThreads);
+        }
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < kUpdItems; ++u)
+        if (id[u] < nmax) s[u] = __ldg(stamp + id[u]);
+#pragma unroll
+    for (uint32_t u = 0; u < kUpdItems; ++u)
+        if (id[u] < nmax && s[u] == ((epoch << 32) | (i0 + u * kUpdThreads))) pos[id[u]] = v[u];
 }
 
 void launch_apply_updates(cudaStream_t st, const uint32_t *ids, const float2 *xy, uint32_t n,
                           uint32_t nmax, unsigned long long epoch, unsigned long long *stamp,
                           float2 *pos, unsigned long long *err) {
     if (n == 0) return;
-    const int T = 256;
-    uint32_t g = (n + T - 1) / T;
-    stamp_kernel<<<g, T, 0, st>>>(ids, n, nmax, epoch, stamp, err);
-    write_winner_kernel<<<g, T, 0, st>>>(ids, xy, n, nmax, epoch, stamp, pos);
+    const uint32_t per = kUpdThreads * kUpdItems, g = n / per + (n % per ? 1u : 0u);
+    stamp_kernel<<<g, kUpdThreads, 0, st>>>(ids, n, nmax, epoch, stamp, err);
+    write_winner_kernel<<<g, kUpdThreads, 0, st>>>(ids, xy, n, nmax, epoch, stamp, pos);
 }
 
 // Object state snapshots (checkpoint / restart): the present flags of the
