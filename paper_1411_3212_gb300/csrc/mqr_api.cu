@@ -109,9 +109,9 @@ struct mqr_ctx {
     DevBuf<uint32_t> sub_q, sub_leaf, sub_len, sub_res, isub, bitmap, item_leaf;
     DevBuf<unsigned long long> out_off;
     // query splitting: coarse lookup table, per-query cells, (query, block) pairs
-    DevBuf<uint32_t> zmap, pair_q, pair_first, pair_blo, pair_rec, qpair, tile_p0;
+    DevBuf<uint32_t> zmap, pair_rec, qpair, tile_p0;
+    DevBuf<uint4> pairs;
     DevBuf<uint2> qcells;
-    DevBuf<unsigned long long> cand_off, pair_off;
     unsigned long long cand_tiles = 0;
     // zero-initialised arena: Info, tile counters, coarse digit counts, look-back status
     DevBuf<unsigned char> arena;
@@ -240,7 +240,7 @@ Arena arena_layout(uint32_t nmax, uint32_t Q, unsigned long long sub_cap, unsign
     Arena a{};
     a.leaf_tiles = (nmax + kLeafTile - 1) / kLeafTile;
     a.lscan_tiles = (nmax + kLeafScanTile - 1) / kLeafScanTile;
-    a.qb_tiles = (Q + kQBQueries - 1) / kQBQueries;
+    a.qb_tiles = (Q + kQBQueries - 1) / kQBQueries;       // (of one step)
     a.cand_tiles = cand_tiles;
     a.res_tiles = (uint32_t)((sub_cap + kResTile - 1) / kResTile) + 1;
     size_t o = 0;
@@ -256,8 +256,9 @@ Arena arena_layout(uint32_t nmax, uint32_t Q, unsigned long long sub_cap, unsign
     a.st_lscan = take((size_t)3 * a.lscan_tiles * sizeof(uint32_t));
     a.st_qb_p = take((size_t)a.qb_tiles * sizeof(uint32_t));
     a.st_qb_c = take((size_t)a.qb_tiles * sizeof(unsigned long long));
-    a.st_cand = take((size_t)((a.cand_tiles + kCandChunkTiles - 1) / kCandChunkTiles + 1) *
-                     sizeof(unsigned long long));
+    // (up to 1,024 chunks of fewer tiles when there are few: see cand_write_kernel)
+    a.st_cand = take((size_t)(std::max<unsigned long long>((a.cand_tiles + kCandChunkTiles - 1) / kCandChunkTiles, 1024) +
+                              1) * sizeof(unsigned long long));
     a.st_res = take((size_t)a.res_tiles * sizeof(unsigned long long));
     a.total = o;
     return a;
@@ -474,16 +475,14 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     phase_begin(c, MQR_PHASE_QUERY_BLOCKS);
     launch_zmap(st, ix->leaf_hi.p, info, c->zmap.p);
     launch_query_blocks(st, rects, Q, x0, y0, c->sx, c->sy, worlds, ix->leaf_lo.p, ix->leaf_hi.p, c->zmap.p,
-                        c->qcells.p, c->cand_off.p, c->pair_q.p, c->pair_first.p, c->pair_blo.p,
-                        c->pair_off.p, c->qpair.p, c->tile_p0.p, a.cand_tiles,
+                        c->qcells.p, c->pairs.p, c->qpair.p, c->tile_p0.p, a.cand_tiles,
                         at<uint32_t>(c, a.st_qb_p), at<unsigned long long>(c, a.st_qb_c), ctr + 5, info);
     phase_end(c, MQR_PHASE_QUERY_BLOCKS, Q ? 2 : 1);
     // a7: candidates -> subquery records
     phase_begin(c, MQR_PHASE_CANDIDATES);
     if (c != ix)      // a slot's per-leaf subquery counts start at zero (the index build zeroes its own)
         MQR_CUDA(cudaMemsetAsync(c->leaf_nsub.p, 0, (size_t)std::max<uint32_t>(nmax, 1) * sizeof(uint32_t), st));
-    launch_candidates(st, c->num_sms * (int)c->bps_cand, cov, c->tile_p0.p, c->pair_q.p, c->pair_first.p, c->pair_blo.p,
-                      c->pair_off.p, c->qcells.p, ix->leaf_box.p, ix->leaf_beg.p, c->leaf_nsub.p, c->pair_rec.p,
+    launch_candidates(st, c->num_sms * (int)c->bps_cand, cov, c->tile_p0.p, c->pairs.p, c->qcells.p, ix->leaf_box.p, ix->leaf_beg.p, c->leaf_nsub.p, c->pair_rec.p,
                       c->sub_q.p, c->sub_leaf.p, c->sub_len.p, c->sub_res.p,
                       at<unsigned long long>(c, a.st_cand), ctr + 8, caps, info);
     phase_end(c, MQR_PHASE_CANDIDATES, 1);
@@ -567,12 +566,8 @@ mqr_status ensure_tick_buffers(mqr_ctx *c, uint32_t Q) {
     size_t sub0 = std::max<size_t>(4096, (size_t)Q * 4);
     MQR_CUDA(c->zmap.ensure(kZCells + 1));
     MQR_CUDA(c->qcells.ensure(std::max<size_t>(Q, 1)));
-    MQR_CUDA(c->cand_off.ensure((size_t)Q + 1));
     MQR_CUDA(c->qpair.ensure((size_t)Q + 1));
-    MQR_CUDA(c->pair_q.ensure((size_t)Q * 9 + 1));
-    MQR_CUDA(c->pair_first.ensure((size_t)Q * 9 + 1));
-    MQR_CUDA(c->pair_blo.ensure((size_t)Q * 9 + 1));
-    MQR_CUDA(c->pair_off.ensure((size_t)Q * 9 + 1));
+    MQR_CUDA(c->pairs.ensure((size_t)Q * 9 + 1));
     MQR_CUDA(c->pair_rec.ensure((size_t)Q * 9 + 2));
     c->cand_tiles = std::min<unsigned long long>(
         std::max<unsigned long long>(c->cand_tiles, std::max<unsigned long long>(1 << 16, 2ull * Q)), kMaxCandTiles);
@@ -1207,13 +1202,11 @@ void mqr_destroy(mqr_ctx *c) {
     DevBuf<uint32_t> *u32s[] = {&c->list_ids, &c->long_lists, &c->skey, &c->sid, &c->sort_counts, &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
                                 &c->leaf_sub_off, &c->leaf_word_off, &c->leaf_item_off,
                                 &c->sub_q, &c->sub_leaf, &c->sub_len, &c->sub_res,
-                                &c->isub, &c->bitmap, &c->item_leaf, &c->up_ids, &c->zmap, &c->pair_q,
-                                &c->pair_first, &c->pair_blo, &c->pair_rec, &c->qpair, &c->tile_p0};
+                                &c->isub, &c->bitmap, &c->item_leaf, &c->up_ids, &c->zmap, &c->pair_rec, &c->qpair, &c->tile_p0};
     for (auto *b : u32s) b->release();
     c->qcells.release();
     c->leaf_box.release();
-    c->cand_off.release();
-    c->pair_off.release();
+    c->pairs.release();
     c->mk_a.release();
     c->mk_b.release();
     c->arena.release();

@@ -371,18 +371,19 @@ constexpr int kZLevel = 8;
 constexpr uint32_t kZCells = 1u << (2 * kZLevel);
 constexpr int kZShift = 2 * (kLevels - kZLevel);
 constexpr int kQBThreads = 256;                       // threads per block of query_blocks
-constexpr int kQBQueries = kQBThreads / 9;            // queries per block (9 block slots each)
+constexpr int kQBQueries = kQBThreads / 9;            // queries of a step (9 block slots each)
+constexpr uint32_t kQBSteps = 2;                      // steps of a block
+constexpr uint32_t kQBOneStep = 32768;                // queries up to which a block takes one step
 constexpr unsigned long long kMaxCandTiles = (1ull << 27) - 1;   // candidates and record indices fit 32 bits
-constexpr int kCandWarpTiles = 8;                     // warp tiles of one warp in one chunk of the candidate pass
+constexpr int kCandWarpTiles = 8;                     // warp tiles of one warp in one chunk of the candidate pass, at most
 constexpr int kCandChunkTiles = 8 * kCandWarpTiles;   // warp tiles of one chunk (a block of 256 threads)
 
 void launch_zmap(cudaStream_t st, const uint32_t *leaf_hi, const Info *info, uint32_t *zmap);
-// a5 + a6: blocks, leaf ranges and candidate counts per query, scanned.
+// a5 + a6: blocks, leaf ranges and candidate counts per query, scanned; a pair is
+// {first candidate, query, first leaf, block corner}.
 void launch_query_blocks(cudaStream_t st, const float4 *rects, uint32_t Q, float x0, float y0, float sx,
                          float sy, Worlds worlds, const uint32_t *leaf_lo, const uint32_t *leaf_hi, const uint32_t *zmap,
-                         uint2 *qcells, unsigned long long *cand_off, uint32_t *pair_q,
-                         uint32_t *pair_first, uint32_t *pair_blo, unsigned long long *pair_off,
-                         uint32_t *qpair, uint32_t *tile_p0, unsigned long long tile_cap,
+                         uint2 *qcells, uint4 *pairs, uint32_t *qpair, uint32_t *tile_p0, unsigned long long tile_cap,
                          uint32_t *status_p, unsigned long long *status_c, uint32_t *tile_counter,
                          Info *info);
 // a7: candidates (warp tiles of 32) -> subquery records (query-major),
@@ -394,14 +395,13 @@ void launch_query_blocks(cudaStream_t st, const float4 *rects, uint32_t Q, float
 // grid only sets how many blocks are resident (mqr_set_launch_config).
 constexpr int kDefaultBlocksPerSM = 8;
 void launch_candidates(cudaStream_t st, int grid_blocks, int covering, const uint32_t *tile_p0,
-                       const uint32_t *pair_q, const uint32_t *pair_first, const uint32_t *pair_blo,
-                       const unsigned long long *pair_off, const uint2 *qcells, const uint2 *leaf_box,
+                       const uint4 *pairs, const uint2 *qcells, const uint2 *leaf_box,
                        const uint32_t *leaf_beg, uint32_t *leaf_nsub, uint32_t *pair_rec, uint32_t *sub_q,
                        uint32_t *sub_leaf, uint32_t *sub_len, uint32_t *sub_res, unsigned long long *status,
                        uint32_t *chunk_counter, Caps caps, Info *info);
 
 // a8: scans over leaves -> leaf_sub_off, leaf_word_off, leaf_item_off, item_leaf.
-constexpr int kLeafScanThreads = 256, kLeafScanItems = 8, kLeafScanTile = kLeafScanThreads * kLeafScanItems;
+constexpr int kLeafScanThreads = 256, kLeafScanItems = 2, kLeafScanTile = kLeafScanThreads * kLeafScanItems;
 void launch_leaf_scan(cudaStream_t st, int num_sms, uint32_t nmax, const uint32_t *leaf_beg,
                       const uint32_t *leaf_nsub, uint32_t *leaf_sub_off, uint32_t *leaf_word_off,
                       uint32_t *leaf_item_off, uint32_t *item_leaf,
