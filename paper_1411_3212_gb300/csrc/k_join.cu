@@ -447,6 +447,17 @@ __device__ __forceinline__ uint4 ld_shared_v4(const uint4 *p) {
 }
 constexpr int kUnitUnroll = 2;           // units whose id loads are issued together
 
+// Start of query q's output: its first record is the first record of its first
+// (query, block) pair (queries without pairs take the next pair's); pair_rec
+// holds that record's index.
+__device__ __forceinline__ unsigned long long query_offset(uint32_t q, uint32_t nsub, uint32_t npairs,
+                                                           const uint32_t *__restrict__ qpair,
+                                                           const uint32_t *__restrict__ pair_rec,
+                                                           const unsigned long long *__restrict__ out_off) {
+    const uint32_t p = qpair[q];
+    return out_off[p < npairs ? pair_rec[p] : nsub];
+}
+
 // One warp per batch of 32 consecutive subquery records (query-major order,
 // so the output is written front to back): lane j loads the metadata of
 // record j into the warp's shared-memory slots; the batch's small
@@ -458,7 +469,7 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
             const uint32_t *__restrict__ sub_len, const uint32_t *__restrict__ leaf_word_off,
             const unsigned long long *__restrict__ out_off, const uint32_t *__restrict__ leaf_beg,
             const uint32_t *__restrict__ sid, const uint32_t *__restrict__ bitmap, void *out,
-            uint32_t wpr, uint32_t *ticket, Caps caps, const Info *info) {
+            uint32_t wpr, uint32_t *ticket, Caps caps, const Info *info, QueryOffsets qo) {
     // per record: {q, bitmap row, first sorted object, objects | covering flag} and its output offset
     __shared__ uint4 s_rec[kEmitWarps][32];
     __shared__ unsigned long long s_off[kEmitWarps][32];
@@ -469,6 +480,11 @@ emit_kernel(const uint32_t *__restrict__ sub_q, const uint32_t *__restrict__ sub
     __shared__ unsigned long long s_uptr[kEmitWarps][32];
     if (!tick_buffers_ok(info, caps)) return;
     uint32_t nsub = (uint32_t)info->n_sub;
+    if (qo.offsets) {           // the per-query offsets, even if the output does not fit
+        const uint32_t npairs = (uint32_t)info->n_pairs;
+        for (uint32_t q = blockIdx.x * kEmitThreads + threadIdx.x; q <= qo.Q; q += gridDim.x * kEmitThreads)
+            qo.offsets[q] = qo.Q && nsub ? query_offset(q, nsub, npairs, qo.qpair, qo.pair_rec, out_off) : 0ull;
+    }
     if (info->emit_end) nsub = min(nsub, (uint32_t)info->emit_end);     // admitted prefix only (low 32 bits)
     if (KIND != kEmitBitmap && out_off[nsub] > caps.out) return;
     const int lane = threadIdx.x & 31;
@@ -593,28 +609,28 @@ void launch_emit(cudaStream_t st, int grid_blocks, int emit_kind, const uint32_t
                  const uint32_t *sub_leaf, const uint32_t *sub_len, const uint32_t *leaf_word_off,
                  const unsigned long long *out_off, const uint32_t *leaf_beg,
                  const uint32_t *sid, const uint32_t *bitmap, void *out, uint32_t wpr,
-                 uint32_t *ticket, Caps caps, const Info *info) {
+                 uint32_t *ticket, Caps caps, const Info *info, const QueryOffsets &qo) {
     const int grid = grid_blocks;
     switch (emit_kind) {
         case kEmitPairs:
             emit_kernel<kEmitPairs><<<grid, kEmitThreads, 0, st>>>(sub_q, sub_leaf, sub_len, leaf_word_off, out_off,
-                                                                   leaf_beg, sid, bitmap, out, wpr, ticket, caps, info);
+                                                                   leaf_beg, sid, bitmap, out, wpr, ticket, caps, info, qo);
             break;
         case kEmitIds:
             emit_kernel<kEmitIds><<<grid, kEmitThreads, 0, st>>>(sub_q, sub_leaf, sub_len, leaf_word_off, out_off,
-                                                                 leaf_beg, sid, bitmap, out, wpr, ticket, caps, info);
+                                                                 leaf_beg, sid, bitmap, out, wpr, ticket, caps, info, qo);
             break;
         case kEmitBitmap:
             emit_kernel<kEmitBitmap><<<grid, kEmitThreads, 0, st>>>(sub_q, sub_leaf, sub_len, leaf_word_off, out_off,
-                                                                    leaf_beg, sid, bitmap, out, wpr, ticket, caps, info);
+                                                                    leaf_beg, sid, bitmap, out, wpr, ticket, caps, info, qo);
             break;
         case kEmitRuns:
             emit_kernel<kEmitRuns><<<grid, kEmitThreads, 0, st>>>(sub_q, sub_leaf, sub_len, leaf_word_off, out_off,
-                                                                  leaf_beg, sid, bitmap, out, wpr, ticket, caps, info);
+                                                                  leaf_beg, sid, bitmap, out, wpr, ticket, caps, info, qo);
             break;
         default:
             emit_kernel<kEmitKeys64><<<grid, kEmitThreads, 0, st>>>(sub_q, sub_leaf, sub_len, leaf_word_off, out_off,
-                                                                    leaf_beg, sid, bitmap, out, wpr, ticket, caps, info);
+                                                                    leaf_beg, sid, bitmap, out, wpr, ticket, caps, info, qo);
             break;
     }
 }
@@ -622,14 +638,6 @@ void launch_emit(cudaStream_t st, int grid_blocks, int emit_kind, const uint32_t
 // Per-query offsets: the first record of query q is the first record of its
 // first (query, block) pair (queries without pairs take the next pair's);
 // pair_rec holds that record's index.
-__device__ __forceinline__ unsigned long long query_offset(uint32_t q, uint32_t nsub, uint32_t npairs,
-                                                           const uint32_t *__restrict__ qpair,
-                                                           const uint32_t *__restrict__ pair_rec,
-                                                           const unsigned long long *__restrict__ out_off) {
-    const uint32_t p = qpair[q];
-    return out_off[p < npairs ? pair_rec[p] : nsub];
-}
-
 // longest: the longest list's length goes to info->max_list (the sorted kinds
 // choose their sort by it).
 __global__ void query_offsets_kernel(uint32_t Q, const uint32_t *__restrict__ qpair,

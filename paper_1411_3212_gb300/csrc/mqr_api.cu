@@ -522,18 +522,21 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
         launch_admit(st, Q, offsets, out ? out_cap_elems : 0, c->qpair.p, c->pair_rec.p, caps, info);
         phase_end(c, MQR_PHASE_OFFSETS, 2);
     }
-    // a12 + a13
-    if (out != nullptr && emit_kind >= 0) {
+    // a12 + a13, and the per-query offsets on the way (alone where nothing is
+    // emitted or, for the sorted kinds, the longest list is wanted too)
+    const bool emits = out != nullptr && emit_kind >= 0;
+    const bool longest = emit_kind == kEmitIds && out == c->list_ids.p;
+    const QueryOffsets qo{Q, c->qpair.p, c->pair_rec.p, emits && !admit && !longest ? offsets : nullptr};
+    if (emits) {
         phase_begin(c, MQR_PHASE_EMIT);
         launch_emit(st, c->num_sms * (int)c->bps_emit, emit_kind, c->sub_q.p, c->sub_leaf.p, c->sub_len.p, c->leaf_word_off.p,
                     c->out_off.p, ix->leaf_beg.p, ix->sid.p, c->bitmap.p, out,
-                    bitmap_words_per_row(nmax), ctr + 9, caps, info);
+                    bitmap_words_per_row(nmax), ctr + 9, caps, info, qo);
         phase_end(c, MQR_PHASE_EMIT, 1);
     }
-    if (offsets != nullptr && !admit) {
+    if (offsets != nullptr && !admit && !qo.offsets) {
         phase_begin(c, MQR_PHASE_OFFSETS);
-        launch_query_offsets(st, Q, c->qpair.p, c->pair_rec.p, c->out_off.p, offsets, caps,
-                             emit_kind == kEmitIds && out == c->list_ids.p, info);
+        launch_query_offsets(st, Q, c->qpair.p, c->pair_rec.p, c->out_off.p, offsets, caps, longest, info);
         phase_end(c, MQR_PHASE_OFFSETS, 1);
     }
     return check_launch("tick kernels");
@@ -936,7 +939,7 @@ mqr_status tick_device_impl(mqr_ctx *c, const float *rects_dev, uint32_t Q, int 
     phase_begin(c, MQR_PHASE_EMIT);
     launch_emit(c->stream, c->num_sms * (int)c->bps_emit, by_lists ? kEmitIds : kEmitKeys64, c->sub_q.p, c->sub_leaf.p,
                 c->sub_len.p, c->leaf_word_off.p, c->out_off.p, c->leaf_beg.p, c->sid.p, c->bitmap.p,
-                by_lists ? (void *)c->list_ids.p : (void *)c->sortA.p, wpr, ticket, caps, info);
+                by_lists ? (void *)c->list_ids.p : (void *)c->sortA.p, wpr, ticket, caps, info, QueryOffsets{});
     phase_end(c, MQR_PHASE_EMIT, 1);
     s = check_launch("emit lists");
     if (s != MQR_OK) return s;

@@ -432,11 +432,17 @@ void launch_result_scan(cudaStream_t st, unsigned long long sub_cap, const uint3
 // a12 + a13: emit results in query-major order.
 enum EmitKind { kEmitPairs = 0, kEmitIds = 1, kEmitBitmap = 2, kEmitKeys64 = 3, kEmitRuns = 4,
                 kEmitAtomic = 5 /* the atomic-append baseline (no bitmaps, unordered pairs) */ };
+// qo.offsets (or null): the per-query offsets, written on the way.
+struct QueryOffsets {
+    uint32_t Q;
+    const uint32_t *qpair, *pair_rec;
+    unsigned long long *offsets;
+};
 void launch_emit(cudaStream_t st, int grid_blocks, int emit_kind, const uint32_t *sub_q,
                  const uint32_t *sub_leaf, const uint32_t *sub_len, const uint32_t *leaf_word_off,
                  const unsigned long long *out_off, const uint32_t *leaf_beg,
                  const uint32_t *sid, const uint32_t *bitmap, void *out, uint32_t bitmap_words_per_row,
-                 uint32_t *ticket, Caps caps, const Info *info);
+                 uint32_t *ticket, Caps caps, const Info *info, const QueryOffsets &qo);
 
 // The atomic-append baseline filtering (Alg. 3) and its covering runs.
 void launch_atomic_baseline(cudaStream_t st, int num_sms, const float4 *rects, const float2 *sxy,
