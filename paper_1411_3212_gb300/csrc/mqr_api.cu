@@ -129,6 +129,7 @@ struct mqr_ctx {
     cudaStream_t copy_stream = nullptr;              // device-to-host copies of mqr_tick_host_async
     DevBuf<uint32_t> sid_stage, sid_stage2;          // sorted-id snapshots copied by mqr_get_sorted_async
     cudaEvent_t snap_done = nullptr;
+    cudaEvent_t up_copied = nullptr;                 // the copies of mqr_apply_updates_host
     cudaEvent_t copy_done[2] = {nullptr, nullptr};
     bool copy_pending[2] = {false, false};
     int next_stage = 0;
@@ -1220,6 +1221,7 @@ void mqr_destroy(mqr_ctx *c) {
         if (c->copy_done[b]) { cudaEventSynchronize(c->copy_done[b]); cudaEventDestroy(c->copy_done[b]); }
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     if (c->snap_done) cudaEventDestroy(c->snap_done);
+    if (c->up_copied) cudaEventDestroy(c->up_copied);
     c->sid_stage.release();
     c->sid_stage2.release();
     c->out_stage.release();
@@ -1339,13 +1341,15 @@ mqr_status mqr_apply_updates_host(mqr_ctx *c, const uint32_t *ids_host, const fl
     MQR_CUDA(cudaSetDevice(c->device));
     MQR_CUDA(c->up_ids.ensure(n));
     MQR_CUDA(c->up_xy.ensure(n));
+    if (!c->up_copied) MQR_CUDA(cudaEventCreateWithFlags(&c->up_copied, cudaEventDisableTiming));
     MQR_CUDA(cudaMemcpyAsync(c->up_ids.p, ids_host, (size_t)n * 4, cudaMemcpyHostToDevice, c->stream));
     MQR_CUDA(cudaMemcpyAsync(c->up_xy.p, xy_host, (size_t)n * 8, cudaMemcpyHostToDevice, c->stream));
+    MQR_CUDA(cudaEventRecord(c->up_copied, c->stream));
     mqr_status s = mqr_apply_updates(c, c->up_ids.p, reinterpret_cast<const float *>(c->up_xy.p), n);
-    if (s != MQR_OK) return s;
-    // the host buffers may be reused as soon as we return
-    MQR_CUDA(cudaStreamSynchronize(c->stream));
-    return MQR_OK;
+    // the host buffers may be reused as soon as we return: wait for their
+    // copies, not for the update kernels behind them
+    MQR_CUDA(cudaEventSynchronize(c->up_copied));
+    return s;
 }
 
 static bool slots_busy(const mqr_ctx *c) {
