@@ -61,73 +61,83 @@ filter_kernel(const float4 *__restrict__ rects, const float2 *__restrict__ sxy,
     const uint32_t items = (uint32_t)info->n_items;
     const int lane = threadIdx.x & 31;
     const float qnan = __int_as_float(0x7fc00000);
-    // items are handed out by a ticket counter (their sizes vary: 1-32
-    // subqueries x 1-8 words) after every warp's first one, which is its own;
-    // the next ticket is drawn during the current item
+    // Items are handed out by a ticket counter (their sizes vary: 1-32
+    // subqueries x 1-8 words), G consecutive ones to a ticket, after every
+    // warp's first group, which is its own; the next ticket is drawn during the
+    // current group.  One word gives out one ticket a nanosecond, which bound
+    // the kernel at one item each: 63,000 items of 4 words 51 -> 31 us, 251,000
+    // of 37 words 205 -> 175, 16,400 of 22 words 20.5 -> 16.5.  Two at a time
+    // keep the balance; four only for many small items (4 words: 33 us with
+    // two; 66 words: 182 with four, 178 with two).
     const uint32_t warps = gridDim.x * (kFilterThreads / 32);
-    uint32_t item = blockIdx.x * (kFilterThreads / 32) + (threadIdx.x >> 5), next = 0xffffffffu;
-    for (; item < items; item = __shfl_sync(0xffffffffu, next, 0)) {
-        if (lane == 0 && items > warps) next = warps + atomicAdd(ticket, 1u);
-        const uint32_t leaf = __ldg(item_leaf + item);
-        const uint32_t r = item - __ldg(leaf_item_off + leaf);
-        const uint32_t soff = __ldg(leaf_sub_off + leaf);
-        const uint32_t nsub = __ldg(leaf_sub_off + leaf + 1) - soff;
-        const uint32_t beg = __ldg(leaf_beg + leaf);
-        const uint32_t nobj = __ldg(leaf_beg + leaf + 1) - beg;
-        const uint32_t ngroups = (nsub + 31u) >> 5;
-        const uint32_t c = r / ngroups, g = r - c * ngroups;
-        const uint32_t nchunk = (nobj + 255u) >> 8;
-        const uint32_t nw_leaf = (nobj + 31u) >> 5;
-        const uint32_t obase = beg + c * 256u;
-        const uint32_t ocnt = min(256u, nobj - c * 256u);
-        const uint32_t nwc = (ocnt + 31u) >> 5;
+    const uint32_t G = items >= 4u * warps && info->n_words < 16ull * items ? 4u : 2u;
+    const uint32_t groups = (items + G - 1u) / G;
+    uint32_t group = blockIdx.x * (kFilterThreads / 32) + (threadIdx.x >> 5), next = 0xffffffffu;
+    for (; group < groups; group = __shfl_sync(0xffffffffu, next, 0)) {
+        if (lane == 0 && groups > warps) next = warps + atomicAdd(ticket, 1u);
+        const uint32_t last = min(items, (group + 1u) * G);
+        for (uint32_t item = group * G; item < last; ++item) {
+            const uint32_t leaf = __ldg(item_leaf + item);
+            const uint32_t r = item - __ldg(leaf_item_off + leaf);
+            const uint32_t soff = __ldg(leaf_sub_off + leaf);
+            const uint32_t nsub = __ldg(leaf_sub_off + leaf + 1) - soff;
+            const uint32_t beg = __ldg(leaf_beg + leaf);
+            const uint32_t nobj = __ldg(leaf_beg + leaf + 1) - beg;
+            const uint32_t ngroups = (nsub + 31u) >> 5;
+            const uint32_t c = r / ngroups, g = r - c * ngroups;
+            const uint32_t nchunk = (nobj + 255u) >> 8;
+            const uint32_t nw_leaf = (nobj + 31u) >> 5;
+            const uint32_t obase = beg + c * 256u;
+            const uint32_t ocnt = min(256u, nobj - c * 256u);
+            const uint32_t nwc = (ocnt + 31u) >> 5;
 
-        float x[8], y[8];
-#pragma unroll
-        for (int wd = 0; wd < 8; ++wd) {
-            uint32_t idx = wd * 32 + lane;
-            if (idx < ocnt) {
-                float2 p = __ldg(sxy + obase + idx);
-                x[wd] = p.x;
-                y[wd] = p.y;
-            } else {
-                x[wd] = qnan;
-                y[wd] = qnan;
-            }
-        }
-        const uint32_t s0 = g * 32u;
-        const uint32_t ns = min(32u, nsub - s0);
-        uint32_t myk = 0;
-        float4 myr = make_float4(qnan, qnan, qnan, qnan);
-        if ((uint32_t)lane < ns) {
-            myk = __ldg(isub + soff + s0 + lane);
-            myr = __ldg(rects + __ldg(sub_q + myk));
-        }
-        uint32_t w[8];
-#pragma unroll
-        for (int wd = 0; wd < 8; ++wd) w[wd] = 0;
-        switch (nwc) {                      // the chunk's word count, fixed per item
-            case 1: filter_words<1>(x, y, myr, ns, lane, w); break;
-            case 2: filter_words<2>(x, y, myr, ns, lane, w); break;
-            case 3: filter_words<3>(x, y, myr, ns, lane, w); break;
-            case 4: filter_words<4>(x, y, myr, ns, lane, w); break;
-            case 5: filter_words<5>(x, y, myr, ns, lane, w); break;
-            case 6: filter_words<6>(x, y, myr, ns, lane, w); break;
-            case 7: filter_words<7>(x, y, myr, ns, lane, w); break;
-            default: filter_words<8>(x, y, myr, ns, lane, w); break;
-        }
-        if ((uint32_t)lane < ns) {
-            uint32_t cnt = 0;
-            const uint32_t row = __ldg(leaf_word_off + leaf) + (s0 + lane) * nw_leaf + c * 8u;
+            float x[8], y[8];
 #pragma unroll
             for (int wd = 0; wd < 8; ++wd) {
-                if ((uint32_t)wd < nwc) {
-                    bitmap[row + wd] = w[wd];
-                    cnt += __popc(w[wd]);
+                uint32_t idx = wd * 32 + lane;
+                if (idx < ocnt) {
+                    float2 p = __ldg(sxy + obase + idx);
+                    x[wd] = p.x;
+                    y[wd] = p.y;
+                } else {
+                    x[wd] = qnan;
+                    y[wd] = qnan;
                 }
             }
-            if (nchunk == 1) sub_res[myk] = cnt;
-            else atomicAdd(sub_res + myk, cnt);
+            const uint32_t s0 = g * 32u;
+            const uint32_t ns = min(32u, nsub - s0);
+            uint32_t myk = 0;
+            float4 myr = make_float4(qnan, qnan, qnan, qnan);
+            if ((uint32_t)lane < ns) {
+                myk = __ldg(isub + soff + s0 + lane);
+                myr = __ldg(rects + __ldg(sub_q + myk));
+            }
+            uint32_t w[8];
+#pragma unroll
+            for (int wd = 0; wd < 8; ++wd) w[wd] = 0;
+            switch (nwc) {                      // the chunk's word count, fixed per item
+                case 1: filter_words<1>(x, y, myr, ns, lane, w); break;
+                case 2: filter_words<2>(x, y, myr, ns, lane, w); break;
+                case 3: filter_words<3>(x, y, myr, ns, lane, w); break;
+                case 4: filter_words<4>(x, y, myr, ns, lane, w); break;
+                case 5: filter_words<5>(x, y, myr, ns, lane, w); break;
+                case 6: filter_words<6>(x, y, myr, ns, lane, w); break;
+                case 7: filter_words<7>(x, y, myr, ns, lane, w); break;
+                default: filter_words<8>(x, y, myr, ns, lane, w); break;
+            }
+            if ((uint32_t)lane < ns) {
+                uint32_t cnt = 0;
+                const uint32_t row = __ldg(leaf_word_off + leaf) + (s0 + lane) * nw_leaf + c * 8u;
+#pragma unroll
+                for (int wd = 0; wd < 8; ++wd) {
+                    if ((uint32_t)wd < nwc) {
+                        bitmap[row + wd] = w[wd];
+                        cnt += __popc(w[wd]);
+                    }
+                }
+                if (nchunk == 1) sub_res[myk] = cnt;
+                else atomicAdd(sub_res + myk, cnt);
+            }
         }
     }
 }
