@@ -516,7 +516,7 @@ def run_gpu(args, name):
     peak, peak_kind = read_peaks()
     achieved = per_launch_bytes / (per_launch_ms / 1000.0) / 1e9 if per_launch_ms > 0 else 0.0
     kernel_names = {"emit": "emit_kernel", "filter": "filter_kernel",
-                    "sort": "tile_hist_kernel+digit_scan_kernel+onesweep_kernel",
+                    "sort": "tile_hist_kernel+group_scan_kernel+sort_pass_kernel (small_sort_kernel: keys and sort)",
                     "query_blocks": "zmap_kernel+query_blocks_kernel", "candidates": "cand_write_kernel",
                     "group": "leaf_scan_kernel+leaf_lists_kernel",
                     "leaves": "leaves_kernel", "keys": "morton_kernel", "updates": "stamp_kernel+write_winner_kernel",

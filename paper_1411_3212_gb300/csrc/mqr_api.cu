@@ -903,7 +903,8 @@ mqr_status tick_device_impl(mqr_ctx *c, const float *rects_dev, uint32_t Q, int 
     MQR_CUDA(c->list_ids.ensure(4096));
     MQR_CUDA(c->long_lists.ensure((size_t)Q + 2));
     const SortedOut so{out_dev, as_pairs};
-    const unsigned long long fits = out_dev ? std::min<unsigned long long>(c->list_ids.n, cap_bytes / eb) : 0;
+    const unsigned long long fits =
+        out_dev ? std::min<unsigned long long>({c->list_ids.n, cap_bytes / eb, (1ull << 30) - 1}) : 0;
     mqr_status s = run_tick(c, rects, Q, kEmitIds, c->list_ids.p, fits, offs, false, &so);
     *out_count = c->last.n_results;
     if (s != MQR_OK) return s;
