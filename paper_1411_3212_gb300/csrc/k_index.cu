@@ -234,7 +234,7 @@ void launch_morton_keys(cudaStream_t st, const float2 *pos, const unsigned long 
 // independent loads); above, group_scan_kernel turns the group rows into
 // starts first, so that a tile never reads more than kSortGroup rows.
 //
-// Measured, all four passes with their counts (start: tile counts, a scan
+// Measured, all four passes with their counts (before: tile counts, a scan
 // kernel per digit over the tiles, match-any ranking): 0.089 -> 0.061 ms at
 // 1M objects, 0.209 -> 0.149 ms at 4M, 0.534 -> 0.367 ms at 12M.
 // ---------------------------------------------------------------------------
