@@ -711,7 +711,7 @@ mqr_status attempt_check(mqr_ctx *c, uint32_t Q, int emit_kind, const Caps &caps
     c->last = in;
     c->last_q = Q;
     c->last_emit_kind = emit_kind;
-    c->have_tick = true;
+    c->have_tick = false;           // until the records are complete: they may not fit, or go with a failed growth
     c->index_valid = true;
     c->snap_pending = false;
     if (in.err & kErrTimeout) return fail(MQR_ERR_TIMEOUT, "a device-side wait exceeded its deadline");
@@ -748,6 +748,7 @@ mqr_status attempt_check(mqr_ctx *c, uint32_t Q, int emit_kind, const Caps &caps
             *again = true;
         }
     }
+    c->have_tick = !*again;
     return MQR_OK;
 }
 
