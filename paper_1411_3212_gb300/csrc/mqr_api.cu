@@ -564,6 +564,17 @@ mqr_status enqueue_slot(mqr_ctx *c, const float4 *rects, uint32_t Q, int emit_ki
     return enqueue_join(c, ix, rects, Q, emit_kind, out, out_cap_elems, offsets, a, caps, true);
 }
 
+// The arrays of n subquery records.  sub_q comes last: its size stands for all
+// of them (Caps::sub), so it must not exist where another's allocation failed.
+mqr_status ensure_records(mqr_ctx *c, size_t n) {
+    MQR_CUDA(c->sub_leaf.ensure(n));
+    MQR_CUDA(c->sub_len.ensure(n));
+    MQR_CUDA(c->sub_res.ensure(n));
+    MQR_CUDA(c->out_off.ensure(n + 1));
+    MQR_CUDA(c->sub_q.ensure(n));
+    return MQR_OK;
+}
+
 // Make sure every per-tick buffer that depends on Q or on the capacities
 // exists.
 mqr_status ensure_tick_buffers(mqr_ctx *c, uint32_t Q) {
@@ -577,28 +588,18 @@ mqr_status ensure_tick_buffers(mqr_ctx *c, uint32_t Q) {
         std::max<unsigned long long>(c->cand_tiles, std::max<unsigned long long>(1 << 16, 2ull * Q)), kMaxCandTiles);
     MQR_CUDA(c->tile_p0.ensure(c->cand_tiles));
     if (c->sub_q.n == 0) {
-        MQR_CUDA(c->sub_q.ensure(sub0));
-        MQR_CUDA(c->sub_leaf.ensure(sub0));
-        MQR_CUDA(c->sub_len.ensure(sub0));
-        MQR_CUDA(c->sub_res.ensure(sub0));
-        MQR_CUDA(c->out_off.ensure(sub0 + 1));
         MQR_CUDA(c->isub.ensure(sub0));
         MQR_CUDA(c->bitmap.ensure(std::max<size_t>(1 << 16, (size_t)Q * 16)));
         MQR_CUDA(c->item_leaf.ensure(std::max<size_t>(1 << 16, (size_t)Q)));
+        return ensure_records(c, sub0);
     }
     return MQR_OK;
 }
 
 mqr_status grow_sub(mqr_ctx *c, unsigned long long need) {
-    size_t n = grow_to(need);
     c->sub_q.release(); c->sub_leaf.release(); c->sub_len.release(); c->sub_res.release();
     c->out_off.release();
-    MQR_CUDA(c->sub_q.ensure(n));
-    MQR_CUDA(c->sub_leaf.ensure(n));
-    MQR_CUDA(c->sub_len.ensure(n));
-    MQR_CUDA(c->sub_res.ensure(n));
-    MQR_CUDA(c->out_off.ensure(n + 1));
-    return MQR_OK;
+    return ensure_records(c, grow_to(need));
 }
 
 // Enqueue the tick's kernels, or, in graph mode (and without phase timing),
