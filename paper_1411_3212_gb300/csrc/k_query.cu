@@ -477,17 +477,22 @@ void launch_candidates(cudaStream_t st, int grid_blocks, int covering, const uin
 // subqueries: its subquery list starts at leaf_sub_off[l]; its bitmap (s rows
 // of ceil(n/32) words, row-major: the linearized layout of Sec. 5.4) starts
 // at leaf_word_off[l]; its filter work items (ceil(n/256) object chunks x
-// ceil(s/32) subquery groups) start at leaf_item_off[l].
+// ceil(s/32) subquery groups) start at leaf_item_off[l].  All sums are 64-bit
+// (one pile of 4M objects and 10,000 subqueries are 1.25e9 words): the totals
+// are exact, and a tick whose words or items pass the limits is refused by the
+// host, the kernels behind this one doing nothing (tick_buffers_ok).  The three
+// offsets, stored in 32 bits, are used only below the limits.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kLeafScanThreads)
 leaf_scan_kernel(const uint32_t *__restrict__ leaf_beg, const uint32_t *__restrict__ leaf_nsub,
                  uint32_t *__restrict__ leaf_sub_off, uint32_t *__restrict__ leaf_word_off,
                  uint32_t *__restrict__ leaf_item_off,
-                 uint32_t *__restrict__ item_leaf, uint32_t *status3, uint32_t num_tiles,
+                 uint32_t *__restrict__ item_leaf, LeafScanSum *status3, uint32_t num_tiles,
                  uint32_t *tile_counter, Caps caps, Info *info) {
     constexpr int NW = kLeafScanThreads / 32;
-    __shared__ uint3 s_warp[NW];
-    __shared__ uint32_t s_tile, s_p[3];
+    __shared__ unsigned long long s_warp[NW][3];
+    __shared__ uint32_t s_tile;
+    __shared__ unsigned long long s_p[3];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t L = (uint32_t)info->n_leaves;
     // tiles of 512 leaves (of 2,048: 8 tiles for 16,384 leaves, 14 us against
@@ -501,43 +506,59 @@ leaf_scan_kernel(const uint32_t *__restrict__ leaf_beg, const uint32_t *__restri
         if (base >= L) break;
         const uint32_t lb = base + tid * kLeafScanItems;
 
-        uint32_t ns[kLeafScanItems], nw[kLeafScanItems], ni[kLeafScanItems];
-        uint32_t t_s = 0, t_w = 0, t_i = 0;
+        uint32_t ns[kLeafScanItems];
+        LeafWork lw[kLeafScanItems];
+        unsigned long long t_s = 0, t_w = 0, t_i = 0;
         unsigned long long objs = 0, tests = 0;
 #pragma unroll
         for (int e = 0; e < kLeafScanItems; ++e) {
             uint32_t l = lb + e;
-            ns[e] = nw[e] = ni[e] = 0;
+            ns[e] = 0;
+            lw[e] = {0, 0};
             if (l < L) {
                 uint32_t sq = leaf_nsub[l];
                 uint32_t n = leaf_beg[l + 1] - leaf_beg[l];
                 ns[e] = sq;
-                nw[e] = sq * ((n + 31u) >> 5);
-                ni[e] = sq ? ((n + 255u) >> 8) * ((sq + 31u) >> 5) : 0u;
+                lw[e] = leaf_work(n, sq);
                 if (sq) objs += (unsigned long long)n * ((sq + 31u) >> 5);
                 tests += (unsigned long long)n * sq;                 // containment tests of the leaf
             }
-            t_s += ns[e]; t_w += nw[e]; t_i += ni[e];
+            t_s += ns[e]; t_w += lw[e].words; t_i += lw[e].items;
         }
-        // one block scan of the three counts together
-        uint32_t i_s = warp_incl_scan(t_s), i_w = warp_incl_scan(t_w), i_i = warp_incl_scan(t_i);
-        if (lane == 31) s_warp[warp] = make_uint3(i_s, i_w, i_i);
+        // one block scan of the three counts together (32-bit inside a warp unless
+        // they are enormous; items never outnumber words)
+        unsigned long long i_s, i_w, i_i;
+        if (__any_sync(0xffffffffu, (t_s | t_w) >= (1ull << 26))) {
+            i_s = warp_incl_scan(t_s);
+            i_w = warp_incl_scan(t_w);
+            i_i = warp_incl_scan(t_i);
+        } else {
+            i_s = warp_incl_scan((uint32_t)t_s);
+            i_w = warp_incl_scan((uint32_t)t_w);
+            i_i = warp_incl_scan((uint32_t)t_i);
+        }
+        if (lane == 31) {
+            s_warp[warp][0] = i_s;
+            s_warp[warp][1] = i_w;
+            s_warp[warp][2] = i_i;
+        }
         objs = warp_sum(objs);
         tests = warp_sum(tests);
         if (lane == 0 && objs) atomicAdd(&info->n_item_objs, objs);
         if (lane == 0 && tests) atomicAdd(&info->n_tests, tests);
         __syncthreads();
-        uint32_t w_s = 0, w_w = 0, w_i = 0, tot_s = 0, tot_w = 0, tot_i = 0;
+        unsigned long long w_s = 0, w_w = 0, w_i = 0, tot_s = 0, tot_w = 0, tot_i = 0;
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
-            const uint3 v = s_warp[w];
-            if (w < warp) { w_s += v.x; w_w += v.y; w_i += v.z; }
-            tot_s += v.x; tot_w += v.y; tot_i += v.z;
+            const unsigned long long v_s = s_warp[w][0], v_w = s_warp[w][1], v_i = s_warp[w][2];
+            if (w < warp) { w_s += v_s; w_w += v_w; w_i += v_i; }
+            tot_s += v_s; tot_w += v_w; tot_i += v_i;
         }
-        uint32_t o_s = w_s + i_s - t_s, o_w = w_w + i_w - t_w, o_i = w_i + i_i - t_i;
+        unsigned long long o_s = w_s + i_s - t_s, o_w = w_w + i_w - t_w, o_i = w_i + i_i - t_i;
         if (tid < 96) {
-            const uint32_t agg = warp == 0 ? tot_s : (warp == 1 ? tot_w : tot_i);
-            const uint32_t pre = lookback_warp<uint32_t>(status3 + (size_t)warp * num_tiles, tile, agg, &info->err);
+            const unsigned long long agg = warp == 0 ? tot_s : (warp == 1 ? tot_w : tot_i);
+            const unsigned long long pre =
+                lookback_warp<LeafScanSum>(status3 + (size_t)warp * num_tiles, tile, agg, &info->err);
             if (lane == 0) s_p[warp] = pre;
         }
         __syncthreads();
@@ -546,18 +567,18 @@ leaf_scan_kernel(const uint32_t *__restrict__ leaf_beg, const uint32_t *__restri
         for (int e = 0; e < kLeafScanItems; ++e) {
             uint32_t l = lb + e;
             if (l < L) {
-                leaf_sub_off[l] = o_s;
-                leaf_word_off[l] = o_w;
-                leaf_item_off[l] = o_i;
-                for (uint32_t t = 0; t < ni[e]; ++t)
-                    if (o_i + t < caps.items) item_leaf[o_i + t] = l;
+                leaf_sub_off[l] = (uint32_t)o_s;
+                leaf_word_off[l] = (uint32_t)o_w;
+                leaf_item_off[l] = (uint32_t)o_i;
+                const unsigned long long end = min(o_i + lw[e].items, caps.items);
+                for (unsigned long long t = o_i; t < end; ++t) item_leaf[t] = l;
             }
-            o_s += ns[e]; o_w += nw[e]; o_i += ni[e];
+            o_s += ns[e]; o_w += lw[e].words; o_i += lw[e].items;
         }
         if (tid == 0 && base + kLeafScanTile >= L) {
-            leaf_sub_off[L] = s_p[0] + tot_s;
-            leaf_word_off[L] = s_p[1] + tot_w;
-            leaf_item_off[L] = s_p[2] + tot_i;
+            leaf_sub_off[L] = (uint32_t)(s_p[0] + tot_s);
+            leaf_word_off[L] = (uint32_t)(s_p[1] + tot_w);
+            leaf_item_off[L] = (uint32_t)(s_p[2] + tot_i);
             info->n_words = s_p[1] + tot_w;
             info->n_items = s_p[2] + tot_i;
         }
@@ -568,7 +589,7 @@ leaf_scan_kernel(const uint32_t *__restrict__ leaf_beg, const uint32_t *__restri
 void launch_leaf_scan(cudaStream_t st, int num_sms, uint32_t nmax, const uint32_t *leaf_beg,
                       const uint32_t *leaf_nsub, uint32_t *leaf_sub_off, uint32_t *leaf_word_off,
                       uint32_t *leaf_item_off, uint32_t *item_leaf,
-                      uint32_t *status3, uint32_t *tile_counter, Caps caps, Info *info) {
+                      LeafScanSum *status3, uint32_t *tile_counter, Caps caps, Info *info) {
     if (nmax == 0) return;
     uint32_t tiles = (nmax + kLeafScanTile - 1) / kLeafScanTile;
     const uint32_t grid = std::min<uint32_t>(tiles, (uint32_t)num_sms * 2u);

@@ -254,7 +254,7 @@ Arena arena_layout(uint32_t nmax, uint32_t Q, unsigned long long sub_cap, unsign
     a.counters = take(16 * sizeof(uint32_t));
     a.sort_group = take(4 * sort_group_words(nmax) * sizeof(uint32_t));   // a set per pass
     a.st_leaf = take((size_t)a.leaf_tiles * sizeof(uint32_t));
-    a.st_lscan = take((size_t)3 * a.lscan_tiles * sizeof(uint32_t));
+    a.st_lscan = take((size_t)3 * a.lscan_tiles * sizeof(LeafScanSum));
     a.st_qb_p = take((size_t)a.qb_tiles * sizeof(uint32_t));
     a.st_qb_c = take((size_t)a.qb_tiles * sizeof(unsigned long long));
     // (up to 1,024 chunks of fewer tiles when there are few: see cand_write_kernel)
@@ -469,7 +469,8 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     // a5 + a6: coarse lookup table, blocks and candidate counts per query
     caps.sub = c->sub_q.n;
     caps.sub_i = c->isub.n;
-    caps.words = std::min<size_t>(c->bitmap.n, 0xffffffffull);
+    // (the atomic baseline builds no bitmaps)
+    caps.words = emit_kind == kEmitAtomic ? ~0ull : std::min<unsigned long long>(c->bitmap.n, kMaxWords);
     caps.out = out_cap_elems;
     caps.cand_tiles = a.cand_tiles;
     caps.items = c->item_leaf.n;
@@ -491,7 +492,7 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     // then every intersecting record into its leaf's list
     phase_begin(c, MQR_PHASE_GROUP);
     launch_leaf_scan(st, c->num_sms, nmax, ix->leaf_beg.p, c->leaf_nsub.p, c->leaf_sub_off.p, c->leaf_word_off.p,
-                     c->leaf_item_off.p, c->item_leaf.p, at<uint32_t>(c, a.st_lscan), ctr + 6, caps, info);
+                     c->leaf_item_off.p, c->item_leaf.p, at<LeafScanSum>(c, a.st_lscan), ctr + 6, caps, info);
     launch_leaf_lists(st, c->num_sms * (int)c->bps_compact, c->sub_leaf.p, c->sub_len.p, c->leaf_sub_off.p,
                       c->isub.p, caps, info);
     phase_end(c, MQR_PHASE_GROUP, nmax ? 2 : 1);
@@ -718,10 +719,14 @@ mqr_status attempt_check(mqr_ctx *c, uint32_t Q, int emit_kind, const Caps &caps
     if (in.err & kErrTimeout) return fail(MQR_ERR_TIMEOUT, "a device-side wait exceeded its deadline");
     if (in.err & kErrInternal) return fail(MQR_ERR_INTERNAL, "device index out of range");
     if (in.err & kErrBadId) c->bad_id = true;
+    switch (tick_limit(in, emit_kind != kEmitAtomic)) {
+        case kTickCandidates:
+            return fail(MQR_ERR_INVALID_ARG, "too many candidate leaves in one tick (limit 2^32)");
+        case kTickWords: return fail(MQR_ERR_CAPACITY, "more than 2^32 bitmap words in one tick");
+        case kTickFits: break;
+    }
     const unsigned long long need_tiles = (in.n_cand + 31) / 32;
     if (need_tiles > caps.cand_tiles) {
-        if (need_tiles > kMaxCandTiles)
-            return fail(MQR_ERR_INVALID_ARG, "too many candidate leaves in one tick (limit 2^32)");
         c->cand_tiles = std::min<unsigned long long>(grow_to(need_tiles), kMaxCandTiles);
         c->tile_p0.release();
         MQR_CUDA(c->tile_p0.ensure(c->cand_tiles));
@@ -742,8 +747,6 @@ mqr_status attempt_check(mqr_ctx *c, uint32_t Q, int emit_kind, const Caps &caps
             *again = true;
         }
         if (in.n_words > caps.words) {
-            if (in.n_words > 0xffffffffull)
-                return fail(MQR_ERR_CAPACITY, "more than 2^32 bitmap words in one tick");
             c->bitmap.release();
             MQR_CUDA(c->bitmap.ensure(grow_to(in.n_words)));
             *again = true;
@@ -927,7 +930,7 @@ mqr_status tick_device_impl(mqr_ctx *c, const float *rects_dev, uint32_t Q, int 
         MQR_CUDA(c->sortB.ensure(R));
     }
     Arena a = arena_layout(c->nmax, Q, c->sub_q.n, c->cand_tiles);
-    Caps caps{c->sub_q.n, c->isub.n, std::min<size_t>(c->bitmap.n, 0xffffffffull), R, c->cand_tiles,
+    Caps caps{c->sub_q.n, c->isub.n, std::min<unsigned long long>(c->bitmap.n, kMaxWords), R, c->cand_tiles,
               c->item_leaf.n};
     Info *info = at<Info>(c, a.info);
     if (by_lists && R <= fits) {                     // only the long lists are left

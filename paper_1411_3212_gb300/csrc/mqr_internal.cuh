@@ -58,6 +58,16 @@ struct Info {
     unsigned long long max_list;     // sorted kinds: the longest query's results
 };
 
+// Filter work of one leaf with n objects and sq intersecting subqueries: its
+// bitmap words (sq rows of ceil(n/32)) and its work items (256 objects x 32
+// subqueries).  Both pass 32 bits long before n or sq does.
+struct LeafWork {
+    unsigned long long words, items;
+};
+__host__ __device__ __forceinline__ LeafWork leaf_work(uint32_t n, uint32_t sq) {
+    return {(unsigned long long)sq * ((n + 31u) >> 5), (unsigned long long)((n + 255u) >> 8) * ((sq + 31u) >> 5)};
+}
+
 // Capacities of the growable per-tick buffers (host-chosen, passed by value).
 struct Caps {
     unsigned long long sub;      // subquery records
@@ -223,6 +233,18 @@ template <> struct StatusBits<unsigned long long> {
     static constexpr unsigned long long kMask = (1ull << 62) - 1;
 };
 
+// A status word and its parts (flag 1: a tile's own sum, 2: the sum up to and
+// with it).  Sums must stay below 2^30 (32-bit words: leaves, of which there are
+// fewer than 2^30 objects) or 2^62.
+template <typename T>
+__host__ __device__ __forceinline__ T status_word(unsigned flag, T sum) {
+    return (T(flag) << StatusBits<T>::kShift) | sum;
+}
+template <typename T>
+__host__ __device__ __forceinline__ unsigned status_flag(T v) { return (unsigned)(v >> StatusBits<T>::kShift); }
+template <typename T>
+__host__ __device__ __forceinline__ T status_sum(T v) { return v & StatusBits<T>::kMask; }
+
 __device__ __forceinline__ uint32_t status_load(const uint32_t *p) {
     return *(const volatile uint32_t *)p;
 }
@@ -239,13 +261,12 @@ __device__ __forceinline__ void status_store(unsigned long long *p, unsigned lon
 template <typename T>
 __device__ T lookback_warp(T *status, uint32_t tile, T agg, unsigned long long *err,
                            unsigned long long wait_ns = kWaitNs) {
-    using B = StatusBits<T>;
     const int lane = threadIdx.x & 31;
     if (tile == 0) {
-        if (lane == 0) status_store(status, (T(2) << B::kShift) | agg);
+        if (lane == 0) status_store(status, status_word<T>(2, agg));
         return T(0);
     }
-    if (lane == 0) status_store(status + tile, (T(1) << B::kShift) | agg);
+    if (lane == 0) status_store(status + tile, status_word<T>(1, agg));
     T sum = 0;
     long j = (long)tile - 1;
     unsigned long long t0 = 0;
@@ -253,9 +274,9 @@ __device__ T lookback_warp(T *status, uint32_t tile, T agg, unsigned long long *
     bool expired = false;
     for (;;) {
         const long idx = j - lane;
-        T v = idx < 0 ? (T(2) << B::kShift) : status_load(status + idx);
+        T v = idx < 0 ? status_word<T>(2, T(0)) : status_load(status + idx);
         for (;;) {
-            const bool inval = (v >> B::kShift) == 0;
+            const bool inval = status_flag(v) == 0;
             if (!__any_sync(0xffffffffu, inval)) break;
             __nanosleep(64);
             if (inval) v = status_load(status + idx);
@@ -273,8 +294,8 @@ __device__ T lookback_warp(T *status, uint32_t tile, T agg, unsigned long long *
             if (lane == 0) atomicOr(err, kErrTimeout);
             break;
         }
-        const T flag = v >> B::kShift, val = v & B::kMask;
-        const uint32_t incl = __ballot_sync(0xffffffffu, flag == 2);
+        const T val = status_sum(v);
+        const uint32_t incl = __ballot_sync(0xffffffffu, status_flag(v) == 2);
         if (incl) {
             const int first = __ffs(incl) - 1;
             sum += warp_sum(lane <= first ? val : T(0));
@@ -283,7 +304,7 @@ __device__ T lookback_warp(T *status, uint32_t tile, T agg, unsigned long long *
         sum += warp_sum(val);
         j -= 32;
     }
-    if (lane == 0) status_store(status + tile, (T(2) << B::kShift) | (sum + agg));
+    if (lane == 0) status_store(status + tile, status_word<T>(2, sum + agg));
     return sum;
 }
 
@@ -375,6 +396,17 @@ constexpr int kQBQueries = kQBThreads / 9;            // queries of a step (9 bl
 constexpr uint32_t kQBSteps = 2;                      // steps of a block
 constexpr uint32_t kQBOneStep = 32768;                // queries up to which a block takes one step
 constexpr unsigned long long kMaxCandTiles = (1ull << 27) - 1;   // candidates and record indices fit 32 bits
+
+// What a tick's totals (64-bit, exact whatever the buffers held) rule out.
+// Word and item indices are 32-bit; the filter counts items in groups of up to
+// four past the last one.  Only kinds that build bitmaps have words.
+constexpr unsigned long long kMaxWords = 0xffffffffull, kMaxItems = 0xffffff00ull;
+enum TickLimit { kTickFits, kTickCandidates, kTickWords };
+inline TickLimit tick_limit(const Info &in, bool bitmaps) {
+    if ((in.n_cand + 31) / 32 > kMaxCandTiles) return kTickCandidates;
+    if (in.n_items > kMaxItems || (bitmaps && in.n_words > kMaxWords)) return kTickWords;
+    return kTickFits;
+}
 constexpr int kCandWarpTiles = 8;                     // warp tiles of one warp in one chunk of the candidate pass, at most
 constexpr int kCandChunkTiles = 8 * kCandWarpTiles;   // warp tiles of one chunk (a block of 256 threads)
 
@@ -401,11 +433,12 @@ void launch_candidates(cudaStream_t st, int grid_blocks, int covering, const uin
                        uint32_t *chunk_counter, Caps caps, Info *info);
 
 // a8: scans over leaves -> leaf_sub_off, leaf_word_off, leaf_item_off, item_leaf.
+using LeafScanSum = unsigned long long;      // records, words and items of all leaves together
 constexpr int kLeafScanThreads = 256, kLeafScanItems = 2, kLeafScanTile = kLeafScanThreads * kLeafScanItems;
 void launch_leaf_scan(cudaStream_t st, int num_sms, uint32_t nmax, const uint32_t *leaf_beg,
                       const uint32_t *leaf_nsub, uint32_t *leaf_sub_off, uint32_t *leaf_word_off,
                       uint32_t *leaf_item_off, uint32_t *item_leaf,
-                      uint32_t *status3, uint32_t *tile_counter, Caps caps, Info *info);
+                      LeafScanSum *status3, uint32_t *tile_counter, Caps caps, Info *info);
 
 // a8: the intersecting records into their leaves' lists (isub).
 void launch_leaf_lists(cudaStream_t st, int grid_blocks, const uint32_t *sub_leaf, const uint32_t *sub_len,
