@@ -116,19 +116,22 @@ __device__ __forceinline__ int classify(uint32_t i0, uint32_t i1, uint32_t j0, u
 // a5 + a6: per query, its blocks and their leaf ranges ("pairs") and the
 // number of candidate leaves; single-pass scans give pair and candidate
 // offsets (the paper's two-pass count / exclusive scan / write scheme, with
-// the write of the pair records fused after the scan).
+// the write of the pair records fused after the scan).  The pairs are summed in
+// 64 bits (up to nine for each of 2^30 queries) and their indices stored in 32:
+// in an answered tick they do not outnumber its candidates, which fit.
 // ---------------------------------------------------------------------------
 template <int M>
 __global__ void __launch_bounds__(kQBThreads, 8)
 query_blocks_kernel(const float4 *__restrict__ rects, uint32_t Q, float x0, float y0, float sx, float sy,
                     Worlds worlds, const uint32_t *__restrict__ leaf_lo, const uint32_t *__restrict__ leaf_hi,
                     const uint32_t *__restrict__ zmap, uint2 *__restrict__ qcells,
-                    uint4 *__restrict__ pairs, uint32_t *__restrict__ qpair, uint32_t *__restrict__ tile_p0, unsigned long long tile_cap, uint32_t *status_p,
-                    unsigned long long *status_c, uint32_t *tile_counter, Info *info) {
+                    uint4 *__restrict__ pairs, uint32_t *__restrict__ qpair, uint32_t *__restrict__ tile_p0,
+                    unsigned long long tile_cap, PairSum *status_p, unsigned long long *status_c,
+                    uint32_t *tile_counter, Info *info) {
     // one thread per (query, block slot): M times kQBQueries queries x 9 slots per block
     constexpr int NW = kQBThreads / 32;
     static_assert(NW * M <= 32, "one warp adds up the warps");
-    __shared__ uint32_t s_wp[NW * M];          // pairs of each warp and step, then of all before it
+    __shared__ PairSum s_wp[NW * M];           // pairs of each warp and step, then of all before it
     __shared__ unsigned long long s_wc[NW * M];
     __shared__ uint32_t s_tile;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -197,13 +200,13 @@ query_blocks_kernel(const float4 *__restrict__ rects, uint32_t Q, float x0, floa
     // one warp each adds up the block's steps and warps and looks back over the earlier tiles
     const bool end = (tile + 1) * (uint32_t)(kQBQueries * M) >= Q;
     if (warp == 0) {
-        const uint32_t v = lane < NW * M ? s_wp[lane] : 0u;
+        const uint32_t v = lane < NW * M ? (uint32_t)s_wp[lane] : 0u;
         const uint32_t inc = warp_incl_scan(v);
         const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
-        const uint32_t pp = lookback_warp<uint32_t>(status_p, tile, tot, &info->err);
-        if (lane < NW * M) s_wp[lane] = pp + inc - v;
+        const PairSum pp = lookback_warp<PairSum>(status_p, tile, tot, &info->err);
+        if (lane < NW * M) s_wp[lane] = pp + (inc - v);
         if (lane == 0 && end) {
-            qpair[Q] = pp + tot;
+            qpair[Q] = (uint32_t)(pp + tot);
             info->n_pairs = pp + tot;
         }
     } else if (warp == 1) {
@@ -220,15 +223,15 @@ query_blocks_kernel(const float4 *__restrict__ rects, uint32_t Q, float x0, floa
 #pragma unroll
     for (int m = 0; m < M; ++m) {
         const uint32_t q = q0 + m * kQBQueries;
-        const uint32_t p = s_wp[m * NW + warp] + __popc(has[m] & lanemask_lt());
+        const PairSum p = s_wp[m * NW + warp] + __popc(has[m] & lanemask_lt());
         const unsigned long long co = s_wc[m * NW + warp] + (inc_c[m] - cnt[m]);
-        if (ql < (uint32_t)kQBQueries && q < Q && slot == 0) qpair[q] = p;
+        if (ql < (uint32_t)kQBQueries && q < Q && slot == 0) qpair[q] = (uint32_t)p;
         if (cnt[m]) {
             pairs[p] = make_uint4((uint32_t)co, q, f[m], blk[m]);
             // warp tiles of 32 candidates whose first candidate falls in this pair
             if (co < (tile_cap << 5)) {             // tile_cap <= 2^27: the tiles fit 32 bits
                 const unsigned long long last = min((co + cnt[m] + 31ull) >> 5, tile_cap);
-                for (uint32_t t = (uint32_t)((co + 31ull) >> 5); t < (uint32_t)last; ++t) tile_p0[t] = p;
+                for (uint32_t t = (uint32_t)((co + 31ull) >> 5); t < (uint32_t)last; ++t) tile_p0[t] = (uint32_t)p;
             }
         }
     }
@@ -241,7 +244,7 @@ void launch_zmap(cudaStream_t st, const uint32_t *leaf_hi, const Info *info, uin
 void launch_query_blocks(cudaStream_t st, const float4 *rects, uint32_t Q, float x0, float y0, float sx,
                          float sy, Worlds worlds, const uint32_t *leaf_lo, const uint32_t *leaf_hi, const uint32_t *zmap,
                          uint2 *qcells, uint4 *pairs, uint32_t *qpair, uint32_t *tile_p0, unsigned long long tile_cap,
-                         uint32_t *status_p, unsigned long long *status_c, uint32_t *tile_counter,
+                         PairSum *status_p, unsigned long long *status_c, uint32_t *tile_counter,
                          Info *info) {
     if (Q == 0) return;
     // two steps a block overlap their loads and halve the tiles to look back

@@ -255,7 +255,7 @@ Arena arena_layout(uint32_t nmax, uint32_t Q, unsigned long long sub_cap, unsign
     a.sort_group = take(4 * sort_group_words(nmax) * sizeof(uint32_t));   // a set per pass
     a.st_leaf = take((size_t)a.leaf_tiles * sizeof(uint32_t));
     a.st_lscan = take((size_t)3 * a.lscan_tiles * sizeof(LeafScanSum));
-    a.st_qb_p = take((size_t)a.qb_tiles * sizeof(uint32_t));
+    a.st_qb_p = take((size_t)a.qb_tiles * sizeof(PairSum));
     a.st_qb_c = take((size_t)a.qb_tiles * sizeof(unsigned long long));
     // (up to 1,024 chunks of fewer tiles when there are few: see cand_write_kernel)
     a.st_cand = take((size_t)(std::max<unsigned long long>((a.cand_tiles + kCandChunkTiles - 1) / kCandChunkTiles, 1024) +
@@ -478,7 +478,7 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     launch_zmap(st, ix->leaf_hi.p, info, c->zmap.p);
     launch_query_blocks(st, rects, Q, x0, y0, c->sx, c->sy, worlds, ix->leaf_lo.p, ix->leaf_hi.p, c->zmap.p,
                         c->qcells.p, c->pairs.p, c->qpair.p, c->tile_p0.p, a.cand_tiles,
-                        at<uint32_t>(c, a.st_qb_p), at<unsigned long long>(c, a.st_qb_c), ctr + 5, info);
+                        at<PairSum>(c, a.st_qb_p), at<unsigned long long>(c, a.st_qb_c), ctr + 5, info);
     phase_end(c, MQR_PHASE_QUERY_BLOCKS, Q ? 2 : 1);
     // a7: candidates -> subquery records
     phase_begin(c, MQR_PHASE_CANDIDATES);

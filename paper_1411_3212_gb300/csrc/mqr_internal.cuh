@@ -413,10 +413,11 @@ constexpr int kCandChunkTiles = 8 * kCandWarpTiles;   // warp tiles of one chunk
 void launch_zmap(cudaStream_t st, const uint32_t *leaf_hi, const Info *info, uint32_t *zmap);
 // a5 + a6: blocks, leaf ranges and candidate counts per query, scanned; a pair is
 // {first candidate, query, first leaf, block corner}.
+using PairSum = unsigned long long;
 void launch_query_blocks(cudaStream_t st, const float4 *rects, uint32_t Q, float x0, float y0, float sx,
                          float sy, Worlds worlds, const uint32_t *leaf_lo, const uint32_t *leaf_hi, const uint32_t *zmap,
                          uint2 *qcells, uint4 *pairs, uint32_t *qpair, uint32_t *tile_p0, unsigned long long tile_cap,
-                         uint32_t *status_p, unsigned long long *status_c, uint32_t *tile_counter,
+                         PairSum *status_p, unsigned long long *status_c, uint32_t *tile_counter,
                          Info *info);
 // a7: candidates (warp tiles of 32) -> subquery records (query-major),
 // placed in one pass (chunks of tiles in ticket order, a look-back over the

@@ -32,6 +32,12 @@ static LeafScanSum *scan_status(void (*)(cudaStream_t, int, uint32_t, const uint
     return nullptr;
 }
 
+static PairSum *pair_status(void (*)(cudaStream_t, const float4 *, uint32_t, float, float, float, float, Worlds,
+                                     const uint32_t *, const uint32_t *, const uint32_t *, uint2 *, uint4 *, uint32_t *,
+                                     uint32_t *, u64, PairSum *, u64 *, uint32_t *, Info *)) {
+    return nullptr;
+}
+
 int main() {
     int bad = 0;
     // a leaf's words and items
@@ -46,6 +52,10 @@ int main() {
     const u64 pile[] = {1250000000ull, 176000000ull, 3000000000ull, 0ull, 1ull << 40};
     (void)scan_status(launch_leaf_scan);                  // the kernel's status words are these
     CHECK(prefixes_hold<LeafScanSum>(pile, 5));
+    // and so do nine pairs of each of up to 2^30 queries
+    const u64 pairs[] = {9ull * 119304648, 9ull * 119304648, 9ull * 400000000, 0ull, 504ull};
+    (void)pair_status(launch_query_blocks);
+    CHECK(prefixes_hold<PairSum>(pairs, 5) && !prefixes_hold<uint32_t>(pairs, 1));
     const u64 leaves[] = {2048, 0, (1u << 30) - 2049};     // leaves: fewer than 2^30
     CHECK(prefixes_hold<uint32_t>(leaves, 3));
     CHECK(!prefixes_hold<uint32_t>(pile, 1));              // why 32-bit words do not do
