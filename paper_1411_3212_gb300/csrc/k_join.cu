@@ -173,13 +173,13 @@ result_scan_kernel(const uint32_t *__restrict__ sub_res, const uint32_t *__restr
     if (!tick_buffers_ok(info, caps)) return;
     const uint32_t tile = s_tile;
     const uint32_t nsub = (uint32_t)info->n_sub;
-    const uint32_t base = tile * kResTile;
+    const unsigned long long base = res_tile_begin(tile);
     if (base >= nsub) {
         if (tile == 0 && tid == 0) out_off[0] = 0;
         return;
     }
-    const uint32_t kb = base + tid * kResItems;
-    const bool whole = kb + kResItems <= nsub;      // the thread's records are all present: vector loads
+    const uint32_t kb = (uint32_t)base + tid * kResItems;
+    const bool whole = res_items_whole(kb, nsub);   // the thread's records are all present: vector loads
     uint32_t rr[kResItems], ll[kResItems];
     if (whole) {
         static_assert(kResItems == 8, "two 16-byte loads per array");

@@ -457,6 +457,15 @@ void launch_filter(cudaStream_t st, int grid_blocks, const float4 *rects, const 
 // withholds its look-back status and the other tiles wait kStallWaitNs only,
 // so their bounded waits run out and the tick reports a timeout.
 constexpr int kResThreads = 256, kResItems = 8, kResTile = kResThreads * kResItems;
+// The first record of a tile (there may be tiles past 2^32: the grid covers the
+// capacity, which grows beyond the records), and whether all of a thread's
+// records, from kb on, are among the first nsub.
+__host__ __device__ __forceinline__ unsigned long long res_tile_begin(uint32_t tile) {
+    return (unsigned long long)tile * kResTile;
+}
+__host__ __device__ __forceinline__ bool res_items_whole(uint32_t kb, uint32_t nsub) {
+    return kb < nsub && nsub - kb >= (uint32_t)kResItems;
+}
 constexpr unsigned long long kStallWaitNs = 1000000ull;   // 1 ms
 void launch_result_scan(cudaStream_t st, unsigned long long sub_cap, const uint32_t *sub_res,
                         const uint32_t *sub_leaf, unsigned long long *out_off,

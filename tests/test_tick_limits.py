@@ -81,6 +81,16 @@ int main() {
     CHECK(tick_limit(in, true) == kTickFits);
     in.n_cand += 1;
     CHECK(tick_limit(in, true) == kTickCandidates);
+    // the result scan's tiles: none past the records starts at one of them, and
+    // no thread of the last tile takes records past the last
+    CHECK(res_tile_begin((1u << 21) + 5) == (1ull << 32) + 5 * (u64)kResTile);
+    const uint32_t most = (uint32_t)(kMaxCandTiles * 32), last = most / kResTile * kResTile;
+    CHECK(res_tile_begin(most / kResTile) == last && most - last < (uint32_t)kResTile);
+    for (uint32_t nsub : {most, most - 8, most - 31, 2048u, 2049u, 7u, 8u})
+        for (uint32_t t = 0; t < (uint32_t)kResThreads; ++t) {
+            const uint32_t kb = (nsub - 1) / kResTile * kResTile + t * kResItems;
+            CHECK(res_items_whole(kb, nsub) == ((u64)kb + kResItems <= nsub));
+        }
     return bad;
 }
 """
