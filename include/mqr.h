@@ -178,8 +178,11 @@ mqr_status mqr_config_default(mqr_config *cfg);
 mqr_status mqr_create(mqr_rect bounds, uint32_t leaf_cap, uint32_t max_objects, mqr_ctx **out);
 
 /* As mqr_create with every knob of mqr_config.  `cuda_stream` is a
- * cudaStream_t the caller owns (NULL: the context creates its own); all work
- * of the context is enqueued on it. */
+ * cudaStream_t the caller owns; all work of the context is enqueued on it.
+ * NULL: the context creates its own, which waits for no other stream, the
+ * default stream included: what a caller's stream writes into a buffer must be
+ * complete before the buffer is passed.  A caller who works on the default
+ * stream passes cudaStreamLegacy (mqr_set_graph too accepts it). */
 mqr_status mqr_create_ex(mqr_rect bounds, const mqr_config *cfg, void *cuda_stream, mqr_ctx **out);
 
 /* Apply position updates (Sec. 2.2 "Batch processing"): object ids_dev[i]

@@ -126,6 +126,7 @@ struct mqr_ctx {
     DevBuf<uint32_t> list_ids, long_lists;
     bool had_long_lists = false;
     DevBuf<unsigned long long> list_off;
+    cudaStream_t capture_stream = nullptr;           // captures of a context on the legacy default stream
     cudaStream_t copy_stream = nullptr;              // device-to-host copies of mqr_tick_host_async
     DevBuf<uint32_t> sid_stage, sid_stage2;          // sorted-id snapshots copied by mqr_get_sorted_async
     cudaEvent_t snap_done = nullptr;
@@ -633,7 +634,17 @@ mqr_status enqueue_or_replay(mqr_ctx *c, const float4 *rects, uint32_t Q, int em
             if (!g.exec || (ge->exec && g.used < ge->used)) ge = &g;
         if (ge->exec) cudaGraphExecDestroy(ge->exec);
         *ge = mqr_ctx::GraphEntry{};
-        MQR_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed));
+        // The legacy default stream cannot be captured: its ticks are captured
+        // on a stream of the context's own and launched on it all the same.
+        const cudaStream_t launch_stream = c->stream;
+        if (launch_stream == cudaStreamLegacy && !c->capture_stream)
+            MQR_CUDA(cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking));
+        if (launch_stream == cudaStreamLegacy) c->stream = c->capture_stream;
+        cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed);
+        if (e != cudaSuccess) {
+            c->stream = launch_stream;
+            return cuda_fail(e, "cudaStreamBeginCapture");
+        }
         std::memset(c->graph_ev_phase, 0, sizeof(c->graph_ev_phase));
         std::memset(c->graph_ev_launches, 0, sizeof(c->graph_ev_launches));
         std::memset(c->graph_launches, 0, sizeof(c->graph_launches));
@@ -641,7 +652,8 @@ mqr_status enqueue_or_replay(mqr_ctx *c, const float4 *rects, uint32_t Q, int em
         mqr_status s = enqueue_tick(c, rects, Q, emit_kind, out, out_cap_elems, offsets, a, caps, false);
         c->capturing = false;
         cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+        e = cudaStreamEndCapture(c->stream, &g);
+        c->stream = launch_stream;
         if (s != MQR_OK) {
             if (g) cudaGraphDestroy(g);
             return s;
@@ -1226,6 +1238,7 @@ void mqr_destroy(mqr_ctx *c) {
     for (int b = 0; b < 2; ++b)
         if (c->copy_done[b]) { cudaEventSynchronize(c->copy_done[b]); cudaEventDestroy(c->copy_done[b]); }
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
+    if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     if (c->snap_done) cudaEventDestroy(c->snap_done);
     if (c->up_copied) cudaEventDestroy(c->up_copied);
     c->sid_stage.release();

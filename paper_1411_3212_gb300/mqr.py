@@ -278,6 +278,12 @@ def mqr_slot_get_stats(slot):
     return s.as_dict()
 
 
+def _handle(stream):
+    """A torch stream as a handle of this library's: torch's default stream has
+    the handle 0, which means a new stream here; cudaStreamLegacy is its name."""
+    return stream.cuda_stream or 1
+
+
 class Slot:
     """A join slot of an Index (mqr_slot_*): answers batches against the
     index's last snapshot on its own CUDA stream (a torch stream: `stream`,
@@ -535,7 +541,10 @@ def mqr_destroy(ctx):
 
 # -- convenience wrapper ------------------------------------------------------
 class Index:
-    """Owns one mqr context; torch tensors in, torch tensors out."""
+    """Owns one mqr context; torch tensors in, torch tensors out.  All its work
+    is enqueued on `stream`, torch's current stream if not given: behind what
+    that stream still has to write into the tensors passed, and before what it
+    does with their memory afterwards."""
 
     def __init__(self, bounds=(0.0, 0.0, 1.0, 1.0), leaf_cap=128, max_objects=1 << 20,
                  index_kind=MQR_INDEX_QUADTREE, grid_level=8, covering=True, stream=None):
@@ -549,7 +558,7 @@ class Index:
         cfg.covering = 1 if covering else 0
         self.max_objects = max_objects
         self.stream = stream if stream is not None else torch.cuda.current_stream()
-        self.ctx = mqr_create_ex(bounds, cfg, ctypes.c_void_p(self.stream.cuda_stream))
+        self.ctx = mqr_create_ex(bounds, cfg, ctypes.c_void_p(_handle(self.stream)))
         self._out = None
 
     def close(self):

@@ -1,0 +1,56 @@
+"""Inputs that torch's stream has yet to write when a call takes them: the
+call's work comes behind the write and before the memory's next use."""
+import numpy as np
+import pytest
+
+from tests.gpu_util import torch_dev
+
+pytestmark = pytest.mark.gpu
+
+N = 50_000
+DELAY = 20_000_000                     # clock cycles: about 10 ms
+
+
+def late(torch, t):
+    """A tensor that holds t once the current stream gets there, zeros before."""
+    out = torch.zeros_like(t)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(DELAY)
+    out.copy_(t)
+    return out
+
+
+def inputs(torch, dev, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    ids = torch.arange(N, dtype=torch.int32, device=dev)
+    xy = torch.rand(N, 2, generator=g, device=dev)
+    corner = torch.rand(2000, 2, generator=g, device=dev)
+    rects = torch.cat([corner, corner + 0.02], 1).contiguous()
+    inside = (xy[None, :, 0] >= rects[:, None, 0]) & (xy[None, :, 0] <= rects[:, None, 2])
+    inside &= (xy[None, :, 1] >= rects[:, None, 1]) & (xy[None, :, 1] <= rects[:, None, 3])
+    counts = inside.sum(1)
+    torch.cuda.synchronize()
+    return ids, xy, rects, counts.cpu().numpy()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("side_stream", [False, True])
+def test_calls_follow_the_current_stream(graph, side_stream):
+    torch, dev = torch_dev()
+    from paper_1411_3212_gb300 import mqr
+    stream = torch.cuda.Stream() if side_stream else torch.cuda.default_stream()
+    with torch.cuda.stream(stream):
+        idx = mqr.Index(leaf_cap=32, max_objects=N)
+        assert idx.stream == stream
+        idx.set_graph(graph)
+        for seed in range(3):
+            ids, xy, rects, counts = inputs(torch, dev, seed)
+            a, b = late(torch, ids), late(torch, xy)
+            idx.apply_updates(a, b)
+            del a, b                                           # the memory's next user writes it later
+            for _ in range(4):
+                torch.empty(N, dtype=torch.int32, device=dev).fill_(-1)
+                torch.empty(N, 2, device=dev).fill_(-1.0)
+            _, offs = idx.tick(late(torch, rects), kind="count")
+            np.testing.assert_array_equal(np.diff(offs.cpu().numpy()), counts)
+        idx.close()
