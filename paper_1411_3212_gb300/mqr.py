@@ -287,20 +287,30 @@ def _handle(stream):
 class Slot:
     """A join slot of an Index (mqr_slot_*): answers batches against the
     index's last snapshot on its own CUDA stream (a torch stream: `stream`,
-    created if not given)."""
+    created if not given).  A join starts behind what torch's current stream
+    still has to write, and its tensors are kept until its end."""
 
     def __init__(self, index, stream=None):
         import torch
         self.index = index
         self.stream = stream if stream is not None else torch.cuda.Stream(device=torch.cuda.current_device())
-        self.slot = mqr_slot_create(index.ctx, ctypes.c_void_p(self.stream.cuda_stream))
+        self.slot = mqr_slot_create(index.ctx, ctypes.c_void_p(_handle(self.stream)))
+        self._current_stream = torch.cuda.current_stream
+        self._tensors = None
 
     def begin(self, rects, kind, out, capacity_bytes, offsets=None):
+        current = self._current_stream()
+        if current != self.stream:
+            self.stream.wait_stream(current)
         mqr_slot_begin(self.slot, rects, int(rects.shape[0]), KINDS[kind] if isinstance(kind, str) else kind,
                        out, capacity_bytes, offsets)
+        self._tensors = (rects, out, offsets)
 
     def end(self):
-        return mqr_slot_end(self.slot)
+        try:
+            return mqr_slot_end(self.slot)
+        finally:
+            self._tensors = None
 
     def stats(self):
         return mqr_slot_get_stats(self.slot)

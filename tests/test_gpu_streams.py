@@ -54,3 +54,37 @@ def test_calls_follow_the_current_stream(graph, side_stream):
             _, offs = idx.tick(late(torch, rects), kind="count")
             np.testing.assert_array_equal(np.diff(offs.cpu().numpy()), counts)
         idx.close()
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_slot_joins_follow_the_current_stream(own_stream):
+    torch, dev = torch_dev()
+    from paper_1411_3212_gb300 import mqr
+    idx = mqr.Index(leaf_cap=32, max_objects=N)
+    slots = [idx.slot(torch.cuda.default_stream() if own_stream and k else None) for k in range(2)]
+    for seed in range(3):
+        ids, xy, rects, counts = inputs(torch, dev, seed)
+        want = np.concatenate([[0], np.cumsum(counts)])
+        a, b = late(torch, ids), late(torch, xy)
+        idx.apply_updates(a, b)
+        idx.snapshot()
+        del a, b
+        outs = []
+        for s in slots:
+            out = torch.empty(2 * int(want[-1]), dtype=torch.int32, device=dev)
+            offs = torch.empty(len(want), dtype=torch.int64, device=dev)
+            s.begin(late(torch, rects), "pairs", out, out.numel() * 4, offs)
+            outs.append(offs)
+            del out, offs                                      # the queries and the output have no other owner
+            for _ in range(4):
+                torch.empty(2000, 4, device=dev).fill_(-1.0)
+                torch.empty(2 * int(want[-1]), dtype=torch.int32, device=dev).fill_(-1)
+        for s, offs in zip(slots, outs):
+            pairs = s._tensors[1]
+            assert s.end() == (2000, int(want[-1])) and s._tensors is None
+            np.testing.assert_array_equal(offs.cpu().numpy(), want)
+            q = pairs.cpu().numpy().reshape(-1, 2)[:, 0]
+            np.testing.assert_array_equal(np.bincount(q, minlength=2000), counts)
+    for s in slots:
+        s.close()
+    idx.close()
