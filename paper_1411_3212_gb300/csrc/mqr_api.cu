@@ -271,6 +271,14 @@ T *at(mqr_ctx *c, size_t off) {
     return reinterpret_cast<T *>(c->arena.p + off);
 }
 
+// Small settings to the device, on the stream that reads them (a copy on the
+// default stream is not ordered with it, and may return before it has ended);
+// waits, so that the host buffer may be reused.
+cudaError_t copy_in(mqr_ctx *c, void *dev, const void *host, size_t bytes) {
+    const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, c->stream);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(c->stream);
+}
+
 mqr_status check_launch(const char *what) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, what);
@@ -1048,9 +1056,9 @@ mqr_status mqr_cost_create(mqr_cost **out) {
     if (e == cudaSuccess) e = m->v.ensure(P);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, m->device);
     if (e == cudaSuccess) e = m->loss.ensure(1);
-    if (e == cudaSuccess) e = cudaMemset(m->params.p, 0, P * 4);
-    if (e == cudaSuccess) e = cudaMemset(m->m.p, 0, P * 4);
-    if (e == cudaSuccess) e = cudaMemset(m->v.p, 0, P * 4);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->params.p, 0, P * 4, m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->m.p, 0, P * 4, m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->v.p, 0, P * 4, m->stream);
     if (e != cudaSuccess) {
         mqr_cost_destroy(m);
         return cuda_fail(e, "mqr_cost_create");
@@ -1063,10 +1071,11 @@ mqr_status mqr_cost_set_params(mqr_cost *m, const float *params_host, uint32_t n
     if (!m || !params_host) return fail(MQR_ERR_INVALID_ARG, "NULL argument");
     if (n_params != cost_param_count()) return fail(MQR_ERR_INVALID_ARG, "wrong parameter count");
     MQR_CUDA(cudaSetDevice(m->device));
-    MQR_CUDA(cudaMemcpy(m->params.p, params_host, (size_t)n_params * 4, cudaMemcpyHostToDevice));
-    MQR_CUDA(cudaMemset(m->m.p, 0, (size_t)n_params * 4));
-    MQR_CUDA(cudaMemset(m->v.p, 0, (size_t)n_params * 4));
+    MQR_CUDA(cudaMemcpyAsync(m->params.p, params_host, (size_t)n_params * 4, cudaMemcpyHostToDevice, m->stream));
+    MQR_CUDA(cudaMemsetAsync(m->m.p, 0, (size_t)n_params * 4, m->stream));
+    MQR_CUDA(cudaMemsetAsync(m->v.p, 0, (size_t)n_params * 4, m->stream));
     m->steps = 0;
+    MQR_CUDA(cudaStreamSynchronize(m->stream));
     return MQR_OK;
 }
 
@@ -1074,8 +1083,8 @@ mqr_status mqr_cost_get_params(mqr_cost *m, float *params_host, uint32_t n_param
     if (!m || !params_host) return fail(MQR_ERR_INVALID_ARG, "NULL argument");
     if (n_params != cost_param_count()) return fail(MQR_ERR_INVALID_ARG, "wrong parameter count");
     MQR_CUDA(cudaSetDevice(m->device));
+    MQR_CUDA(cudaMemcpyAsync(params_host, m->params.p, (size_t)n_params * 4, cudaMemcpyDeviceToHost, m->stream));
     MQR_CUDA(cudaStreamSynchronize(m->stream));
-    MQR_CUDA(cudaMemcpy(params_host, m->params.p, (size_t)n_params * 4, cudaMemcpyDeviceToHost));
     return MQR_OK;
 }
 
@@ -1173,7 +1182,7 @@ mqr_status mqr_set_region_caps(mqr_ctx *c, uint32_t region_bits, const uint32_t 
     MQR_CUDA(cudaStreamSynchronize(c->stream));
     if (region_bits) {
         MQR_CUDA(c->region_cap.ensure(n));
-        MQR_CUDA(cudaMemcpy(c->region_cap.p, caps_host, n * sizeof(uint32_t), cudaMemcpyHostToDevice));
+        MQR_CUDA(copy_in(c, c->region_cap.p, caps_host, n * sizeof(uint32_t)));
     }
     c->region_bits = region_bits;
     ++g_buf_gen;                                   // a captured tick holds the old configuration
@@ -1420,7 +1429,7 @@ mqr_status mqr_set_worlds(mqr_ctx *c, uint32_t n_worlds, const uint32_t *obj_bas
         return fail(MQR_ERR_INVALID_ARG, "uniform grid: grid_level must be >= log4(n_worlds)");
     MQR_CUDA(c->world_obj.ensure((size_t)n_worlds + 1));
     MQR_CUDA(c->world_q.ensure((size_t)n_worlds + 1));
-    MQR_CUDA(cudaMemcpy(c->world_obj.p, obj_base_host, ((size_t)n_worlds + 1) * 4, cudaMemcpyHostToDevice));
+    MQR_CUDA(copy_in(c, c->world_obj.p, obj_base_host, ((size_t)n_worlds + 1) * 4));
     c->n_worlds = n_worlds;
     c->world_bits = bits;
     return MQR_OK;
@@ -1435,7 +1444,7 @@ mqr_status mqr_set_query_worlds(mqr_ctx *c, const uint32_t *q_base_host) {
         if (q_base_host[w + 1] < q_base_host[w]) return fail(MQR_ERR_INVALID_ARG, "q_base must not decrease");
     MQR_CUDA(cudaSetDevice(c->device));
     MQR_CUDA(cudaStreamSynchronize(c->stream));
-    MQR_CUDA(cudaMemcpy(c->world_q.p, q_base_host, ((size_t)c->n_worlds + 1) * 4, cudaMemcpyHostToDevice));
+    MQR_CUDA(copy_in(c, c->world_q.p, q_base_host, ((size_t)c->n_worlds + 1) * 4));
     c->world_q_total = q_base_host[c->n_worlds];
     c->world_q_set = true;
     return MQR_OK;

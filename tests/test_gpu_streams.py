@@ -88,3 +88,30 @@ def test_slot_joins_follow_the_current_stream(own_stream):
     for s in slots:
         s.close()
     idx.close()
+
+
+def test_settings_do_not_depend_on_the_default_stream():
+    """A model and a context's settings while torch's default stream is busy: the first is all zeros until
+    it is given parameters, and both behave as they do with an idle one."""
+    torch, dev = torch_dev()
+    from paper_1411_3212_gb300 import mqr
+    rng = np.random.default_rng(3)
+    X, y = rng.uniform(-1, 1, (40, 5)).astype(np.float32), rng.uniform(-1, 1, 40).astype(np.float32)
+    got = []
+    for busy in (False, True):
+        blocks = [torch.full((1 << 16,), 7.0, device=dev) for _ in range(64)]      # memory that is not zero
+        del blocks
+        torch.cuda.empty_cache()
+        torch.cuda.synchronize()
+        if busy:
+            torch.cuda._sleep(DELAY)
+        m = mqr.CostModel()
+        first = m.predict(X)
+        p = rng.standard_normal(m.P).astype(np.float32) * 0.1 if not busy else got[0][2]
+        m.set_params(p)
+        loss = m.train(X, y, epochs=3, lr=1e-2)
+        got.append((first, loss, p, m.params()))
+        m.close()
+    assert not got[0][0].any() and not got[1][0].any()
+    assert got[0][1] == got[1][1]
+    np.testing.assert_array_equal(got[0][3], got[1][3])
