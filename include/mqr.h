@@ -432,7 +432,8 @@ mqr_status mqr_cost_set_params(mqr_cost *m, const float *params_host, uint32_t n
 mqr_status mqr_cost_get_params(mqr_cost *m, float *params_host, uint32_t n_params);
 /* `epochs` full-batch Adam steps (beta 0.9 / 0.999, eps 1e-8, bias-corrected)
  * of the mean squared error over the n samples X_host[n][5] -> y_host[n];
- * *loss_out (may be NULL) = the loss before the last step.  Blocks. */
+ * *loss_out (may be NULL) = the loss before the last step.  Blocks.  After an
+ * error (INVALID_ARG, OOM, CUDA) the model is as it was. */
 mqr_status mqr_cost_train(mqr_cost *m, const float *X_host, const float *y_host, uint32_t n, uint32_t epochs,
                           float lr, float *loss_out);
 /* The gradient of the mean squared error over the n samples with respect to
@@ -506,6 +507,12 @@ mqr_status mqr_debug_fail_allocation(int after);
  * tick needs more than one scan tile (over 2,048 subquery records) for a
  * wait to happen. */
 mqr_status mqr_debug_stall_scan(int enable);
+
+/* Test hook for training above 256 samples, which runs as a grid whose blocks
+ * wait for one another for a limited time: 1 makes the next such training's
+ * wait run out after 1 ms (one block withholds its arrival); it is then done by
+ * one cluster of blocks, with the same results.  The hook disarms itself; 0 disarms it.  Errors: INVALID_ARG. */
+mqr_status mqr_debug_cost_grid(int mode);
 
 /* Enable (1) or disable (0) per-phase timing; enabling resets the
  * accumulators.  Timing adds two event records per phase to the stream. */

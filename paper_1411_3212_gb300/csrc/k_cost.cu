@@ -18,6 +18,7 @@
 // of short phases, bound by latency and barriers: 400 epochs of 80 samples take
 // 3.9 ms, 100 epochs of 4,096 take 1.5 (40.4 and 393 with one block for all
 // chunks, two shared-memory loads to a multiplication).
+#include <algorithm>
 #include <cstddef>
 
 #include "mqr_internal.cuh"
@@ -233,9 +234,10 @@ __device__ void cost_chunk(CostSmem &sm, const float *__restrict__ X, const floa
 
 // All blocks of the launch: a cluster barrier, or a counter that every block
 // of a cooperative grid raises (the wait gives up after kWaitNs).  Returns
-// false after a wait that ran out.
+// false after a wait that ran out.  stall_test: block 0 withholds its arrival
+// and the wait is kStallWaitNs.
 template <bool CLUSTER>
-__device__ __forceinline__ bool cost_barrier(CostSmem &sm, uint32_t *sync, uint32_t &target) {
+__device__ __forceinline__ bool cost_barrier(CostSmem &sm, uint32_t *sync, uint32_t &target, int stall_test) {
     if (CLUSTER) {
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
         return true;
@@ -244,14 +246,14 @@ __device__ __forceinline__ bool cost_barrier(CostSmem &sm, uint32_t *sync, uint3
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(sync, 1u);
-        const unsigned long long t0 = global_ns();
+        if (!stall_test || blockIdx.x) atomicAdd(sync, 1u);
+        const unsigned long long t0 = global_ns(), limit = stall_test ? kStallWaitNs : kWaitNs;
         uint32_t v;
         int stop = 0;
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(sync) : "memory");
             if ((int)(v - target) >= 0) break;
-            if (global_ns() - t0 > kWaitNs) {
+            if (global_ns() - t0 > limit) {
                 atomicExch(sync + 1, 1u);
                 stop = 1;
                 break;
@@ -266,15 +268,17 @@ __device__ __forceinline__ bool cost_barrier(CostSmem &sm, uint32_t *sync, uint3
 
 // Block b takes chunk r * gridDim + b in round r of an epoch (blocks without
 // one only own parameters) and owns the parameters [b * per, (b + 1) * per),
-// at most kOwn to a thread, whose moments stay in registers.  part: gridDim x
-// kPart floats; grad_acc: the gradients carried from round to round; sync: the
-// barrier's counter and its time-out flag, zeroed before the launch.
+// at most kOwn to a thread, whose moments stay in registers.  The new
+// parameters and moments go to arrays of their own, so a launch whose wait ran
+// out leaves the model as it was.  part: gridDim x kPart floats; grad_acc: the
+// gradients carried from round to round; sync: the barrier's counter and its
+// time-out flag, zeroed before the launch.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(kCostThreads, 1)
-cost_train_kernel(float *params, float *__restrict__ adam_m, float *__restrict__ adam_v, uint32_t step0,
+cost_train_kernel(CostState from, CostState to, uint32_t step0,
                   const float *__restrict__ X, const float *__restrict__ y, uint32_t n, uint32_t epochs, float lr,
                   float *__restrict__ loss_out, float *__restrict__ grad_out, float *part, float *__restrict__ grad_acc,
-                  uint32_t *sync) {
+                  uint32_t *sync, int stall_test) {
     extern __shared__ __align__(16) unsigned char cost_smem[];
     CostSmem &sm = *reinterpret_cast<CostSmem *>(cost_smem);
     float *stage = reinterpret_cast<float *>(cost_smem + sizeof(CostSmem));
@@ -289,11 +293,11 @@ cost_train_kernel(float *params, float *__restrict__ adam_m, float *__restrict__
 #pragma unroll
     for (int q = 0; q < kOwn; ++q) {
         const uint32_t i = i0 + q * kCostThreads + tid;
-        mo[q] = i < i1 ? adam_m[i] : 0.f;
-        vo[q] = i < i1 ? adam_v[i] : 0.f;
-        po[q] = i < i1 ? params[i] : 0.f;
+        mo[q] = i < i1 ? from.m[i] : 0.f;
+        vo[q] = i < i1 ? from.v[i] : 0.f;
+        po[q] = i < i1 ? from.params[i] : 0.f;
     }
-    cost_load_params(sm, params, tid);
+    cost_load_params(sm, from.params, tid);
     __syncthreads();
     float loss = 0.f;                                                           // warp 0 of block 0
     for (uint32_t ep = 0; ep < epochs; ++ep) {
@@ -301,7 +305,7 @@ cost_train_kernel(float *params, float *__restrict__ adam_m, float *__restrict__
         for (uint32_t r = 0; r < rounds; ++r) {
             const uint32_t here = min(blocks, chunks - r * blocks);             // chunks of this round
             if (b < here) cost_chunk(sm, X, y, n, (r * blocks + b) * kCostChunk, part + (size_t)b * kPart, tid);
-            if (!cost_barrier<CLUSTER>(sm, sync, target)) return;
+            if (!cost_barrier<CLUSTER>(sm, sync, target, stall_test)) return;
             // the owned parameters' gradients: their chunks added in order
             float g[kOwn];
 #pragma unroll
@@ -370,15 +374,15 @@ cost_train_kernel(float *params, float *__restrict__ adam_m, float *__restrict__
                         mo[q] = m;
                         vo[q] = v;
                         po[q] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
-                        __stcg(params + i, po[q]);
+                        __stcg(to.params + i, po[q]);
                     }
                 }
             }
             if (grad_out && r + 1 == rounds) return;
-            if (!cost_barrier<CLUSTER>(sm, sync, target)) return;
+            if (!cost_barrier<CLUSTER>(sm, sync, target, stall_test)) return;
         }
         if (!report) {
-            cost_load_params(sm, params, tid);
+            cost_load_params(sm, to.params, tid);
             __syncthreads();
         }
     }
@@ -386,8 +390,8 @@ cost_train_kernel(float *params, float *__restrict__ adam_m, float *__restrict__
     for (int q = 0; q < kOwn; ++q) {
         const uint32_t i = i0 + q * kCostThreads + tid;
         if (i < i1) {
-            adam_m[i] = mo[q];
-            adam_v[i] = vo[q];
+            to.m[i] = mo[q];
+            to.v[i] = vo[q];
         }
     }
 }
@@ -407,30 +411,30 @@ cost_predict_kernel(const float *__restrict__ p, const float *__restrict__ X, ui
     if (tid < cn) out[c0 + tid] = o;
 }
 
+bool cost_train_grid(uint32_t n) { return n > (uint32_t)(kCostClusterMax * kCostChunk); }
+
 // Blocks of a training launch: one per chunk, at least what the owned
-// parameters need; above a cluster, as many rounds as the SMs make necessary.
-static uint32_t cost_blocks(uint32_t n, int num_sms, bool *cluster) {
+// parameters need; in a grid, as many rounds as the SMs make necessary.
+static uint32_t cost_blocks(uint32_t n, int num_sms, bool grid) {
     static_assert(kCostBlocksMin <= kCostClusterMax, "a cluster holds every parameter");
+    if (!grid) return kCostClusterMax;
     const uint32_t chunks = n / kCostChunk + (n % kCostChunk ? 1u : 0u);
-    *cluster = chunks <= (uint32_t)kCostClusterMax;
-    if (*cluster) return kCostClusterMax;
     const uint32_t rounds = (chunks + num_sms - 1) / num_sms;
     return (chunks + rounds - 1) / rounds;
 }
 
 size_t cost_train_scratch_floats(uint32_t n, int num_sms) {
-    bool cluster;
-    return (size_t)(cost_blocks(n, num_sms, &cluster) + 1) * kPart + 64;
+    return (size_t)(std::max<uint32_t>(cost_blocks(n, num_sms, cost_train_grid(n)), kCostClusterMax) + 1) * kPart + 64;
 }
 
 // scratch: cost_train_scratch_floats(n, num_sms) floats: the chunks' gradients,
 // the gradients carried between rounds, the barrier.  *sync_out: the barrier's
-// words ([1] is set if a wait ran out).
-cudaError_t launch_cost_train(cudaStream_t st, int num_sms, float *params, float *m, float *v, uint32_t step0,
-                              const float *X, const float *y, uint32_t n, uint32_t epochs, float lr, float *loss,
-                              float *grad, float *scratch, uint32_t **sync_out) {
-    bool cluster;
-    const uint32_t blocks = cost_blocks(n, num_sms, &cluster);
+// words ([1] is set if a wait ran out: only a grid's can).
+cudaError_t launch_cost_train(cudaStream_t st, int num_sms, bool grid, const CostState &from, const CostState &to,
+                              uint32_t step0, const float *X, const float *y, uint32_t n, uint32_t epochs, float lr,
+                              float *loss, float *grad, float *scratch, uint32_t **sync_out, bool stall_test) {
+    const bool cluster = !grid;
+    const uint32_t blocks = cost_blocks(n, num_sms, grid);
     float *part = scratch, *acc = scratch + (size_t)blocks * kPart;
     uint32_t *sync = reinterpret_cast<uint32_t *>(acc + kPart);
     *sync_out = sync;
@@ -456,10 +460,10 @@ cudaError_t launch_cost_train(cudaStream_t st, int num_sms, float *params, float
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     if (cluster)
-        return cudaLaunchKernelEx(&cfg, cost_train_kernel<true>, params, m, v, step0, X, y, n, epochs, lr, loss, grad,
-                                  part, acc, sync);
-    return cudaLaunchKernelEx(&cfg, cost_train_kernel<false>, params, m, v, step0, X, y, n, epochs, lr, loss, grad,
-                              part, acc, sync);
+        return cudaLaunchKernelEx(&cfg, cost_train_kernel<true>, from, to, step0, X, y, n, epochs, lr, loss, grad,
+                                  part, acc, sync, 0);
+    return cudaLaunchKernelEx(&cfg, cost_train_kernel<false>, from, to, step0, X, y, n, epochs, lr, loss, grad,
+                              part, acc, sync, stall_test ? 1 : 0);
 }
 
 cudaError_t launch_cost_predict(cudaStream_t st, const float *params, const float *X, uint32_t n, float *out) {

@@ -51,6 +51,9 @@ std::atomic<long long> g_fail_alloc_after{-1};
 // runs with a withheld look-back status and a 1 ms wait limit.
 std::atomic<bool> g_stall_scan{false};
 
+// The same for training (mqr_debug_cost_grid): 1 the next grid's barrier runs out.
+std::atomic<int> g_cost_grid{0};
+
 // A device buffer that only grows (contents are not preserved on growth).
 template <typename T>
 struct DevBuf {
@@ -1014,11 +1017,14 @@ struct mqr_cost {
     cudaStream_t stream = nullptr;
     int num_sms = 0;
     DevBuf<float> params, m, v, X, y, out, loss, scratch;
+    DevBuf<float> next[3];          // a training's parameters and moments, the model's when it has ended well
     uint32_t steps = 0;
 };
 
-// One training (or, with grad, gradient) launch and its results: the loss and
-// whether the kernel's barrier ran out of time.
+// One training (or, with grad, gradient) and its loss.  A grid's barrier may
+// run out of time (its blocks do not get on the device together while other
+// work holds it); one cluster then does the same sums.  The model takes over the new state
+// last, so that whatever failed before leaves it as it was.
 static mqr_status cost_run(mqr_cost *m, const float *X_host, const float *y_host, uint32_t n, uint32_t epochs, float lr,
                            float *grad_dev, float *grad_host, float *loss_out) {
     MQR_CUDA(m->X.ensure((size_t)n * 5));
@@ -1026,17 +1032,27 @@ static mqr_status cost_run(mqr_cost *m, const float *X_host, const float *y_host
     MQR_CUDA(m->scratch.ensure(cost_train_scratch_floats(n, m->num_sms)));
     MQR_CUDA(cudaMemcpyAsync(m->X.p, X_host, (size_t)n * 5 * 4, cudaMemcpyHostToDevice, m->stream));
     MQR_CUDA(cudaMemcpyAsync(m->y.p, y_host, (size_t)n * 4, cudaMemcpyHostToDevice, m->stream));
-    uint32_t *sync = nullptr, gave_up[2] = {0, 0};
-    MQR_CUDA(launch_cost_train(m->stream, m->num_sms, m->params.p, m->m.p, m->v.p, m->steps, m->X.p, m->y.p, n, epochs,
-                               lr, m->loss.p, grad_dev, m->scratch.p, &sync));
-    if (!grad_dev) m->steps += epochs;
+    for (auto &b : m->next) MQR_CUDA(b.ensure(cost_param_count()));
+    const CostState from{m->params.p, m->m.p, m->v.p}, to{m->next[0].p, m->next[1].p, m->next[2].p};
     float l = 0.f;
-    if (grad_dev)
-        MQR_CUDA(cudaMemcpyAsync(grad_host, grad_dev, cost_param_count() * 4, cudaMemcpyDeviceToHost, m->stream));
-    MQR_CUDA(cudaMemcpyAsync(&l, m->loss.p, 4, cudaMemcpyDeviceToHost, m->stream));
-    MQR_CUDA(cudaMemcpyAsync(gave_up, sync, sizeof(gave_up), cudaMemcpyDeviceToHost, m->stream));
-    MQR_CUDA(cudaStreamSynchronize(m->stream));
-    if (gave_up[1]) return fail(MQR_ERR_TIMEOUT, "a device-side wait exceeded its deadline");
+    for (bool grid = cost_train_grid(n);; grid = false) {
+        const bool stall = grid && g_cost_grid.exchange(0) == 1;
+        uint32_t *sync = nullptr, gave_up[2] = {0, 0};
+        MQR_CUDA(launch_cost_train(m->stream, m->num_sms, grid, from, to, m->steps, m->X.p, m->y.p, n, epochs, lr,
+                                   m->loss.p, grad_dev, m->scratch.p, &sync, stall));
+        if (grad_dev)
+            MQR_CUDA(cudaMemcpyAsync(grad_host, grad_dev, cost_param_count() * 4, cudaMemcpyDeviceToHost, m->stream));
+        MQR_CUDA(cudaMemcpyAsync(&l, m->loss.p, 4, cudaMemcpyDeviceToHost, m->stream));
+        MQR_CUDA(cudaMemcpyAsync(gave_up, sync, sizeof(gave_up), cudaMemcpyDeviceToHost, m->stream));
+        MQR_CUDA(cudaStreamSynchronize(m->stream));
+        if (!gave_up[1]) break;
+    }
+    if (!grad_dev) {
+        std::swap(m->params, m->next[0]);
+        std::swap(m->m, m->next[1]);
+        std::swap(m->v, m->next[2]);
+        m->steps += epochs;
+    }
     if (loss_out) *loss_out = l;
     return MQR_OK;
 }
@@ -1125,6 +1141,7 @@ void mqr_cost_destroy(mqr_cost *m) {
     if (m->stream) cudaStreamSynchronize(m->stream);
     m->params.release(); m->m.release(); m->v.release(); m->X.release(); m->y.release();
     m->out.release(); m->loss.release(); m->scratch.release();
+    for (auto &b : m->next) b.release();
     if (m->stream) cudaStreamDestroy(m->stream);
     delete m;
 }
@@ -1817,6 +1834,12 @@ mqr_status mqr_result_footprint(mqr_ctx *c, uint64_t *out_host) {
 
 mqr_status mqr_debug_stall_scan(int enable) {
     g_stall_scan.store(enable != 0);
+    return MQR_OK;
+}
+
+mqr_status mqr_debug_cost_grid(int mode) {
+    if (mode < 0 || mode > 1) return fail(MQR_ERR_INVALID_ARG, "mode must be 0 or 1");
+    g_cost_grid.store(mode);
     return MQR_OK;
 }
 

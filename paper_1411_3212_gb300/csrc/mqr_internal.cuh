@@ -223,6 +223,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s
+constexpr unsigned long long kStallWaitNs = 1000000ull;   // 1 ms (the failure-handling test hooks)
 
 template <typename T> struct StatusBits;
 template <> struct StatusBits<uint32_t> {
@@ -466,7 +467,6 @@ __host__ __device__ __forceinline__ unsigned long long res_tile_begin(uint32_t t
 __host__ __device__ __forceinline__ bool res_items_whole(uint32_t kb, uint32_t nsub) {
     return kb < nsub && nsub - kb >= (uint32_t)kResItems;
 }
-constexpr unsigned long long kStallWaitNs = 1000000ull;   // 1 ms
 void launch_result_scan(cudaStream_t st, unsigned long long sub_cap, const uint32_t *sub_res,
                         const uint32_t *sub_leaf, unsigned long long *out_off,
                         unsigned long long *status, uint32_t *tile_counter, uint32_t run_elems, Caps caps, Info *info,
@@ -497,9 +497,16 @@ void launch_atomic_baseline(cudaStream_t st, int num_sms, const float4 *rects, c
 // Learned tick-cost model (k_cost.cu): MLP 5 -> 64 -> 64 -> 1.
 size_t cost_param_count();
 size_t cost_train_scratch_floats(uint32_t n, int num_sms);
-cudaError_t launch_cost_train(cudaStream_t st, int num_sms, float *params, float *m, float *v, uint32_t step0,
-                              const float *X, const float *y, uint32_t n, uint32_t epochs, float lr, float *loss,
-                              float *grad, float *scratch, uint32_t **sync_out);
+bool cost_train_grid(uint32_t n);       // whether a training of n samples is a grid (else one cluster)
+struct CostState {
+    float *params, *m, *v;
+};
+// A training: from's state after `epochs` steps goes to `to` (grad: only the
+// gradient and the loss are written).  Any n may be trained by one cluster too,
+// with the same results: its barrier is the hardware's and always ends.
+cudaError_t launch_cost_train(cudaStream_t st, int num_sms, bool grid, const CostState &from, const CostState &to,
+                              uint32_t step0, const float *X, const float *y, uint32_t n, uint32_t epochs, float lr,
+                              float *loss, float *grad, float *scratch, uint32_t **sync_out, bool stall_test);
 cudaError_t launch_cost_predict(cudaStream_t st, const float *params, const float *X, uint32_t n, float *out);
 
 // Admission by output memory: queries [0, A) whose output fits cap elements.

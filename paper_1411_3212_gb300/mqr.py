@@ -36,7 +36,7 @@ EXPORTS = ["mqr_config_default", "mqr_create", "mqr_create_ex", "mqr_apply_updat
            "mqr_cost_destroy", "mqr_get_stats",
            "mqr_get_leaves",
            "mqr_get_sorted", "mqr_result_footprint", "mqr_export_state", "mqr_import_state",
-           "mqr_debug_fail_allocation", "mqr_debug_stall_scan",
+           "mqr_debug_fail_allocation", "mqr_debug_stall_scan", "mqr_debug_cost_grid",
            "mqr_set_timing", "mqr_set_timing_phases", "mqr_get_timing",
            "mqr_sort_objects_noalloc",
            "mqr_last_error", "mqr_destroy"]
@@ -145,6 +145,7 @@ def load(path: str = LIB_PATH):
         "mqr_import_state": ([P, P, P, u32], i32),
         "mqr_debug_fail_allocation": ([i32], i32),
         "mqr_debug_stall_scan": ([i32], i32),
+        "mqr_debug_cost_grid": ([i32], i32),
         "mqr_result_footprint": ([P, P], i32),
         "mqr_get_timing": ([P, ctypes.POINTER(mqr_timing)], i32),
         "mqr_sort_objects_noalloc": ([mqr_rect, P, u32, P, P, P], i32),
@@ -510,6 +511,10 @@ def mqr_debug_fail_allocation(after):
 
 def mqr_debug_stall_scan(enable=True):
     _check(load().mqr_debug_stall_scan(1 if enable else 0))
+
+
+def mqr_debug_cost_grid(mode):
+    _check(load().mqr_debug_cost_grid(int(mode)))
 
 
 def mqr_result_footprint(ctx):
