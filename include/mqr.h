@@ -510,8 +510,9 @@ mqr_status mqr_debug_stall_scan(int enable);
 
 /* Test hook for training above 256 samples, which runs as a grid whose blocks
  * wait for one another for a limited time: 1 makes the next such training's
- * wait run out after 1 ms (one block withholds its arrival); it is then done by
- * one cluster of blocks, with the same results.  The hook disarms itself; 0 disarms it.  Errors: INVALID_ARG. */
+ * wait run out after 1 ms (one block withholds its arrival), 2 makes its launch
+ * count as refused; either is then done by one cluster of blocks, with the same
+ * results.  The hook disarms itself; 0 disarms it.  Errors: INVALID_ARG. */
 mqr_status mqr_debug_cost_grid(int mode);
 
 /* Enable (1) or disable (0) per-phase timing; enabling resets the

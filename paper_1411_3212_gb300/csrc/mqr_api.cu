@@ -51,7 +51,8 @@ std::atomic<long long> g_fail_alloc_after{-1};
 // runs with a withheld look-back status and a 1 ms wait limit.
 std::atomic<bool> g_stall_scan{false};
 
-// The same for training (mqr_debug_cost_grid): 1 the next grid's barrier runs out.
+// The same for training (mqr_debug_cost_grid): 1 the next grid's barrier runs
+// out, 2 its launch counts as refused.
 std::atomic<int> g_cost_grid{0};
 
 // A device buffer that only grows (contents are not preserved on growth).
@@ -1023,7 +1024,8 @@ struct mqr_cost {
 
 // One training (or, with grad, gradient) and its loss.  A grid's barrier may
 // run out of time (its blocks do not get on the device together while other
-// work holds it); one cluster then does the same sums.  The model takes over the new state
+// work holds it) and its launch may be refused (fewer SMs than the device has);
+// one cluster then does the same sums.  The model takes over the new state
 // last, so that whatever failed before leaves it as it was.
 static mqr_status cost_run(mqr_cost *m, const float *X_host, const float *y_host, uint32_t n, uint32_t epochs, float lr,
                            float *grad_dev, float *grad_host, float *loss_out) {
@@ -1036,10 +1038,16 @@ static mqr_status cost_run(mqr_cost *m, const float *X_host, const float *y_host
     const CostState from{m->params.p, m->m.p, m->v.p}, to{m->next[0].p, m->next[1].p, m->next[2].p};
     float l = 0.f;
     for (bool grid = cost_train_grid(n);; grid = false) {
-        const bool stall = grid && g_cost_grid.exchange(0) == 1;
+        const int hook = grid ? g_cost_grid.exchange(0) : 0;
         uint32_t *sync = nullptr, gave_up[2] = {0, 0};
-        MQR_CUDA(launch_cost_train(m->stream, m->num_sms, grid, from, to, m->steps, m->X.p, m->y.p, n, epochs, lr,
-                                   m->loss.p, grad_dev, m->scratch.p, &sync, stall));
+        const cudaError_t e = hook == 2 ? cudaErrorCooperativeLaunchTooLarge
+                                        : launch_cost_train(m->stream, m->num_sms, grid, from, to, m->steps, m->X.p, m->y.p,
+                                                            n, epochs, lr, m->loss.p, grad_dev, m->scratch.p, &sync, hook == 1);
+        if (grid && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "training launch");
         if (grad_dev)
             MQR_CUDA(cudaMemcpyAsync(grad_host, grad_dev, cost_param_count() * 4, cudaMemcpyDeviceToHost, m->stream));
         MQR_CUDA(cudaMemcpyAsync(&l, m->loss.p, 4, cudaMemcpyDeviceToHost, m->stream));
@@ -1838,7 +1846,7 @@ mqr_status mqr_debug_stall_scan(int enable) {
 }
 
 mqr_status mqr_debug_cost_grid(int mode) {
-    if (mode < 0 || mode > 1) return fail(MQR_ERR_INVALID_ARG, "mode must be 0 or 1");
+    if (mode < 0 || mode > 2) return fail(MQR_ERR_INVALID_ARG, "mode must be 0, 1 or 2");
     g_cost_grid.store(mode);
     return MQR_OK;
 }

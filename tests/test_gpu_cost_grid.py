@@ -23,7 +23,7 @@ def samples(n):
 
 
 @pytest.mark.parametrize("n", [257, 300, 4096, 20001])
-@pytest.mark.parametrize("mode", [1])
+@pytest.mark.parametrize("mode", [1, 2])
 def test_training_without_a_grid_is_the_same(n, mode, hooks):
     torch_dev()
     from paper_1411_3212_gb300 import mqr
