@@ -702,13 +702,14 @@ struct SortedOut {
 
 mqr_status enqueue_list_sort(mqr_ctx *c, uint32_t Q, const unsigned long long *offsets, const SortedOut &so,
                              const Caps &caps, const Info *info, bool short_lists, bool long_lists) {
+    if (Q == 0) return MQR_OK;      // no lists, and the long lists' counters are the last tick's
     phase_begin(c, MQR_PHASE_OUTPUT_SORT);
     if (short_lists)
         MQR_CUDA(launch_list_sort(c->stream, c->list_ids.p, offsets, Q, so.as_pairs, so.out, c->long_lists.p, caps, info));
     if (long_lists)
         MQR_CUDA(launch_long_lists(c->stream, c->num_sms, c->list_ids.p, offsets, so.as_pairs, so.out, c->long_lists.p,
                                    caps, info));
-    phase_end(c, MQR_PHASE_OUTPUT_SORT, (short_lists && Q ? 1 : 0) + (long_lists ? 1 : 0));
+    phase_end(c, MQR_PHASE_OUTPUT_SORT, (short_lists ? 1 : 0) + (long_lists ? 1 : 0));
     return MQR_OK;
 }
 
