@@ -1050,6 +1050,8 @@ cudaError_t launch_region_counts(cudaStream_t st, const uint32_t *skey, uint32_t
     return cudaGetLastError();
 }
 
+static constexpr size_t leaf_tables(uint32_t cap) { return (size_t)19 * (kLeafTile / 8 + (cap + 8) / 8); }
+
 void launch_build_leaves(cudaStream_t st, const uint32_t *skey, uint32_t nmax, uint32_t cap,
                          int uniform_grid, uint32_t grid_level, uint32_t min_level, uint32_t region_bits,
                          const uint32_t *region_cap, uint8_t *mk_a, uint8_t *mk_b,
@@ -1069,7 +1071,9 @@ void launch_build_leaves(cudaStream_t st, const uint32_t *skey, uint32_t nmax, u
     } else if (!uniform_grid && cap < nmax) {
         if (cap <= (uint32_t)kLeafCapSmem) {
             // prefix and suffix maxima of the blocks of 8 positions and three rows of block maxima
-            dyn = (size_t)19 * (kLeafTile / 8 + (cap + 8) / 8);
+            dyn = leaf_tables(cap);
+            static_assert(leaf_tables(kLeafCapSmem) + kLeafTile + 8 + 8 * (1 << (2 * kMaxRegionBits)) + 256 <= 48 * 1024,
+                          "with the kernel's own arrays, what a launch may have without asking for more");
         } else {
             uint32_t size = nmax + cap + 1;   // cap < nmax: fits the 2*nmax+2 buffers
             window_enc_kernel<<<1024, 256, 0, st>>>(skey, cap, size, info, mk_a);
