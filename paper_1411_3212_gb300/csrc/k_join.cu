@@ -68,9 +68,12 @@ filter_kernel(const float4 *__restrict__ rects, const float2 *__restrict__ sxy,
     // the kernel at one item each: 63,000 items of 4 words 51 -> 31 us, 251,000
     // of 37 words 205 -> 175, 16,400 of 22 words 20.5 -> 16.5.  Two at a time
     // keep the balance; four only for many small items (4 words: 33 us with
-    // two; 66 words: 182 with four, 178 with two).
+    // two; 66 words: 182 with four, 178 with two).  While every warp's own item
+    // is all it gets no ticket is drawn, and two would follow one another in
+    // half of the warps (2,459 items of 10 words 10.2 us against 8.2 with one,
+    // 4,421 of 46 words 13.2 against 11.3).
     const uint32_t warps = gridDim.x * (kFilterThreads / 32);
-    const uint32_t G = items >= 4u * warps && info->n_words < 16ull * items ? 4u : 2u;
+    const uint32_t G = items <= warps ? 1u : items >= 4u * warps && info->n_words < 16ull * items ? 4u : 2u;
     const uint32_t groups = (items + G - 1u) / G;
     uint32_t group = blockIdx.x * (kFilterThreads / 32) + (threadIdx.x >> 5), next = 0xffffffffu;
     for (; group < groups; group = __shfl_sync(0xffffffffu, next, 0)) {
