@@ -359,10 +359,12 @@ mqr_status mqr_set_index(mqr_ctx *ctx, int index_kind, uint32_t leaf_cap, uint32
  * pass (which also places the subquery records), the pass that files the
  * intersecting subqueries into their leaves' lists (compact_blocks_per_sm),
  * the filter (Alg. 2) and the decoding / emit (Alg. 4); 0 keeps the default
- * (8).  Their blocks draw work items from
- * counters or stride over them, so the shapes change time, never results;
- * block sizes are fixed per kernel by its register budget.  An autotuner
- * (autotune.tune_launch_config) picks them by timing.  1 <= value <= 64.
+ * (8).  Their blocks draw work items from counters or stride over them (a
+ * filter or emit warp's first item or batch is its own, so the more blocks,
+ * resident or not, the more of the work is handed out in advance), so the
+ * shapes change time, never results; block sizes are fixed per kernel by its
+ * register budget.  An autotuner (autotune.tune_launch_config) picks them by
+ * timing.  1 <= value <= 64.
  * Call between ticks.  Errors: INVALID_ARG. */
 typedef struct {
     uint32_t candidate_blocks_per_sm;
@@ -548,7 +550,7 @@ mqr_status mqr_get_timing(const mqr_ctx *ctx, mqr_timing *out);
  * on a device looks the array's address up (cudaGetSymbolAddress), so make it
  * before any stream capture.  All calls share the array: calls that overlap
  * on the GPU (e.g. on different streams) race.  Blocks until done.  Errors:
- * INVALID_ARG, CUDA, TIMEOUT, INTERNAL.  cuda_stream: a cudaStream_t or NULL. */
+ * INVALID_ARG, CUDA, INTERNAL.  cuda_stream: a cudaStream_t or NULL. */
 mqr_status mqr_sort_objects_noalloc(mqr_rect bounds, const float *xy_dev, uint32_t n,
                                     uint32_t *keys_out_dev, uint32_t *ids_out_dev, void *cuda_stream);
 

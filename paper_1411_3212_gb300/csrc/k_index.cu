@@ -579,7 +579,7 @@ small_sort_kernel(const float2 *__restrict__ pos, const unsigned long long *__re
         reinterpret_cast<uint4 *>(&s_whist[0][0])[tid] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         uint16_t *wh = s_whist[warp];
-        uint32_t r[(ITEMS + 1) / 2];                            // ranks in the warp's keys (at most 512)
+        uint32_t r[(ITEMS + 1) / 2];                            // ranks in the warp's keys (at most 128)
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
             const uint32_t dg = (uint32_t)(k[it] >> shift) & 255u;

@@ -880,8 +880,10 @@ void launch_atomic_baseline(cudaStream_t st, int num_sms, const float4 *rects, c
 // of id and query.  The networks are straight-line code, so instruction fetch
 // binds next to the barriers: lists of 257 to 1,024 ids in a warp (16 and 32
 // keys to a lane) made it 0.46 ms, blocks of 8 or 16 warps 0.43 and 0.57.
-// 30.7M results of 99,991 queries, 63% of them in lists above 1,024: 0.37 ms,
-// against 2.9 for histograms, six passes and the layout of 8-byte keys.
+// 29.9M results of 99,991 queries, 63% of them in lists above 1,024: 0.39 ms,
+// against 1.28 for six passes over 8-byte keys and their layout, which a tick
+// with a longer list still takes (23.6M results, 195 lists above kBlockList:
+// 0.88 ms and a first emit of ids that nothing reads).
 // ---------------------------------------------------------------------------
 constexpr int kListWarps = 4, kLongWarps = 16;
 constexpr uint32_t kWarpList = 8 * 32;

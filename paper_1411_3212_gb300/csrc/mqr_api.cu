@@ -497,8 +497,8 @@ mqr_status enqueue_join(mqr_ctx *c, const mqr_ctx *ix, const float4 *rects, uint
     phase_begin(c, MQR_PHASE_CANDIDATES);
     if (c != ix)      // a slot's per-leaf subquery counts start at zero (the index build zeroes its own)
         MQR_CUDA(cudaMemsetAsync(c->leaf_nsub.p, 0, (size_t)std::max<uint32_t>(nmax, 1) * sizeof(uint32_t), st));
-    launch_candidates(st, c->num_sms * (int)c->bps_cand, cov, c->tile_p0.p, c->pairs.p, c->qcells.p, ix->leaf_box.p, ix->leaf_beg.p, c->leaf_nsub.p, c->pair_rec.p,
-                      c->sub_q.p, c->sub_leaf.p, c->sub_len.p, c->sub_res.p,
+    launch_candidates(st, c->num_sms * (int)c->bps_cand, cov, c->tile_p0.p, c->pairs.p, c->qcells.p, ix->leaf_box.p,
+                      ix->leaf_beg.p, c->leaf_nsub.p, c->pair_rec.p, c->sub_q.p, c->sub_leaf.p, c->sub_len.p, c->sub_res.p,
                       at<unsigned long long>(c, a.st_cand), ctr + 8, caps, info);
     phase_end(c, MQR_PHASE_CANDIDATES, 1);
     // a8: group intersecting subqueries by leaf: the leaves' list offsets,
@@ -840,7 +840,6 @@ mqr_status sort_result_keys(mqr_ctx *c, uint64_t n, uint32_t Q, unsigned long lo
     unsigned long long herr = 0;
     MQR_CUDA(cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, c->stream));
     MQR_CUDA(cudaStreamSynchronize(c->stream));
-    if (herr & kErrTimeout) return fail(MQR_ERR_TIMEOUT, "a device-side wait exceeded its deadline");
     if (herr) return fail(MQR_ERR_INTERNAL, "device index out of range in the result sort");
     return MQR_OK;
 }
@@ -1256,10 +1255,12 @@ void mqr_destroy(mqr_ctx *c) {
     DevBuf<unsigned long long> *u64s[] = {&c->stamp, &c->keysA, &c->keysB, &c->out_off, &c->off_stage,
                                           &c->sortA, &c->sortB, &c->list_off};
     for (auto *b : u64s) b->release();
-    DevBuf<uint32_t> *u32s[] = {&c->list_ids, &c->long_lists, &c->skey, &c->sid, &c->sort_counts, &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
+    DevBuf<uint32_t> *u32s[] = {&c->list_ids, &c->long_lists, &c->skey, &c->sid, &c->sort_counts,
+                                &c->leaf_lo, &c->leaf_hi, &c->leaf_beg, &c->leaf_nsub,
                                 &c->leaf_sub_off, &c->leaf_word_off, &c->leaf_item_off,
                                 &c->sub_q, &c->sub_leaf, &c->sub_len, &c->sub_res,
-                                &c->isub, &c->bitmap, &c->item_leaf, &c->up_ids, &c->zmap, &c->pair_rec, &c->qpair, &c->tile_p0};
+                                &c->isub, &c->bitmap, &c->item_leaf, &c->up_ids, &c->zmap, &c->pair_rec, &c->qpair,
+                                &c->tile_p0};
     for (auto *b : u32s) b->release();
     c->qcells.release();
     c->leaf_box.release();
@@ -1335,13 +1336,14 @@ mqr_status mqr_create_ex(mqr_rect bounds, const mqr_config *cfg, void *cuda_stre
     }
     c->small_sort = c->nmax <= kSmallSortMax && small_sort_ready();
     const size_t n = std::max<size_t>(c->nmax, 1);
-    if ((e = c->pos.ensure(n)) || (e = c->stamp.ensure(n)) || (e = c->keysA.ensure(n)) ||
-        (e = c->keysB.ensure(n)) || (e = c->skey.ensure(n)) || (e = c->sid.ensure(n)) ||
+    const size_t n_passes = c->small_sort ? 0 : n;      // the sort's passes, which the one-launch sort does not run
+    if ((e = c->pos.ensure(n)) || (e = c->stamp.ensure(n)) || (e = c->keysA.ensure(n_passes)) ||
+        (e = c->keysB.ensure(n_passes)) || (e = c->skey.ensure(n)) || (e = c->sid.ensure(n)) ||
         (e = c->sxy.ensure(n)) || (e = c->leaf_lo.ensure(n)) || (e = c->leaf_hi.ensure(n)) ||
         (e = c->leaf_beg.ensure(n + 1)) || (e = c->leaf_nsub.ensure(n)) ||
         (e = c->leaf_sub_off.ensure(n + 1)) || (e = c->leaf_word_off.ensure(n + 1)) ||
         (e = c->leaf_item_off.ensure(n + 1)) ||
-        (e = c->sort_counts.ensure((size_t)256 * sort_tiles((uint32_t)n))) ||
+        (e = c->sort_counts.ensure((size_t)256 * sort_tiles((uint32_t)n_passes))) ||
         (e = c->upd_err.ensure(1)) || (e = c->leaf_box.ensure(n)))
         return bail(e, "cudaMalloc (object state)");
     if (cfg->index_kind == MQR_INDEX_QUADTREE && cfg->leaf_cap > (uint32_t)kLeafCapSmem &&
