@@ -848,6 +848,7 @@ mqr_status sort_result_keys(mqr_ctx *c, uint64_t n, uint32_t Q, unsigned long lo
 // in c->last; waits for a pending snapshot.
 mqr_status index_ready(mqr_ctx *c) {
     if (c->snap_pending) {
+        MQR_CUDA(cudaSetDevice(c->device));         // the default stream is the current device's
         unsigned long long h[4] = {0, 0, 0, 0};
         MQR_CUDA(cudaMemcpyAsync(h, c->snap_info.p, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
         MQR_CUDA(cudaStreamSynchronize(c->stream));
