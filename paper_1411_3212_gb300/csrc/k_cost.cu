@@ -440,7 +440,9 @@ cudaError_t launch_cost_train(cudaStream_t st, int num_sms, bool grid, const Cos
     *sync_out = sync;
     const size_t smem = sizeof(CostSmem) + (blocks > kCostDirect ? (size_t)blocks * kStage * sizeof(float) : 0);
     const void *f = cluster ? (const void *)cost_train_kernel<true> : (const void *)cost_train_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is the kernel's, shared by all threads: always the largest any of its launches needs
+    const size_t most = sizeof(CostSmem) + (cluster ? 0 : (size_t)num_sms * kStage * sizeof(float));
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e == cudaSuccess) e = cudaMemsetAsync(sync, 0, 2 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr{};
